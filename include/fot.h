@@ -55,22 +55,23 @@ typedef enum {
 } fot_status;
 
 typedef enum {
-  FOT_FP32 = 0,          /* FP32 on the CUDA cores, banded: every output sums only the terms
-                            within 2^-40 of its largest (a provable window per 32-output
-                            tile); for large eps the window sum is a tilted FP32 GEMM with
-                            per-row max-offsets, for small eps an exact windowed
+  FOT_FP32 = 0,          /* FP32, banded: every output sums only the terms within 2^-40 of its
+                            largest (a provable window per tile of outputs); where eps allows, the
+                            window sum is a matrix product of FP32 operands with per-row max-offsets
+                            (each product split into three TF32 ones on the tensor cores, 2^-21
+                            relative, accumulated in FP32), for small eps an exact windowed
                             log-sum-exp */
-  FOT_MIXED = 1,         /* the banded GEMM on tcgen05 tensor cores (split-BF16 operands,
-                            FP32 accumulation in TMEM) with FP32 log-domain potentials */
+  FOT_MIXED = 1,         /* the same with split-BF16 operands (three products, 2^-16 relative) and
+                            FP32 log-domain potentials */
   FOT_FP32_DENSE = 2,    /* FP32 on the CUDA cores, every output scans every term with its
                             own exact maximum (one exponential per term): the plain form */
   FOT_AUTO = 3,          /* batches only: time FOT_FP32 and FOT_MIXED on the batch when its
                             graph is built and keep the faster */
-  FOT_BF16 = 4           /* the tensor-core banded GEMM of FOT_MIXED with single BF16
-                            operands: one MMA per term instead of three; each product carries
-                            up to 2^-7 relative error (both operands rounded to 8 significant
-                            bits), so a half-step moves f or psi by at most 2^-6 eps (against
-                            2^-15 eps for FOT_MIXED); single contexts only */
+  FOT_BF16 = 4           /* the banded product of FOT_MIXED with single BF16 operands: one product
+                            per term instead of three, up to 2^-7 relative error each (both
+                            operands rounded to 8 significant bits), so a half-step moves f or psi
+                            by at most 2^-6 eps (against 2^-15 eps for FOT_MIXED); single contexts
+                            only */
 } fot_precision;
 
 typedef enum { FOT_EPS_PX2 = 0, FOT_EPS_PAPER = 1 } fot_eps_units;
@@ -332,22 +333,22 @@ fot_status fot_loop_time(fot_ctx* ctx, double* ms_out, int64_t* passes_out);
 /* Number of (row, output, summation index) terms the axis passes of this context have
  * evaluated since creation: rows*len*len per dense pass, the window sizes for banded passes
  * (each term is one multiply-add of the exp-domain contraction); tensor_terms_out (may be
- * NULL) receives the part computed on the tensor cores (each term there is three BF16
+ * NULL) receives the part computed from BF16 operands (each term there is three BF16
  * multiply-adds of the split-precision product).  Synchronising. */
 fot_status fot_work_count(fot_ctx* ctx, int64_t* terms_out, int64_t* tensor_terms_out);
 
-/* The same count split by where the terms were evaluated: out4[0] banded tilted-GEMM items
- * (CUDA-core FFMA), out4[1] banded exact-window items (one exponential per term), out4[2]
- * tensor cores, out4[3] dense exact passes (including the phase step's moment passes).
+/* The same count split by how the terms were evaluated: out4[0] banded products of FP32
+ * operands, out4[1] banded exact windows (one exponential per term), out4[2] banded products of
+ * BF16 operands, out4[3] dense exact passes (including the phase step's moment passes).
  * Synchronising.  The paper has no counterpart: a measurement aid. */
 fot_status fot_work_split(fot_ctx* ctx, int64_t* out4);
 
 /* Kernel classes of fot_kernel_times. */
 enum {
-  FOT_KERNEL_PLAN = 0,     /* window plan of a banded pass (and the B-operand table of the
-                              tensor-core pass, written when eps changes) */
-  FOT_KERNEL_BAND = 1,     /* banded pass on the CUDA cores (tilted-GEMM and exact-window items) */
-  FOT_KERNEL_TENSOR = 2,   /* tensor-core banded pass */
+  FOT_KERNEL_PLAN = 0,     /* window plan of a banded pass (and the tilt tables of the BF16 forms,
+                              written once per loop) */
+  FOT_KERNEL_BAND = 1,     /* window sums of a banded pass, FP32 operands */
+  FOT_KERNEL_TENSOR = 2,   /* window sums of a banded pass, BF16 operands */
   FOT_KERNEL_DENSE = 3,    /* dense exact pass */
   FOT_KERNEL_CLASSES = 4
 };

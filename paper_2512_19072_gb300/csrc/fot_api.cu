@@ -1,6 +1,6 @@
 // C ABI of the FOT library (include/fot.h): context lifetime, argument checking, the
-// Sinkhorn loop of Algorithm 1 and the phase step, on top of the kernels in fot_simt.cu
-// (exact FP32 passes), fot_tc.cu (tensor-core passes) and fot_ctransform.cu.
+// Sinkhorn loop of Algorithm 1 and the phase step, on top of the kernels in fot_band.cu and
+// fot_window.cuh (banded passes), fot_simt.cu (dense FP32 passes, moments) and fot_ctransform.cu.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -9,7 +9,7 @@
 #include <new>
 #include <vector>
 
-#include "fot_common.cuh"
+#include "fot_band.cuh"
 
 namespace fot {
 void half_step_simt(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
@@ -30,15 +30,10 @@ void marginal_stats(fot_ctx* c, const float* f, const float* S, const float* psi
 void integrate_phase(fot_ctx* c, const float* Dx, const float* Dy, double dx, float* phi);
 void c_transform_envelope(fot_ctx* c, const float* pot_in, float* out);
 void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
-                    float* pot_out, float* logsum, float* tmp);
-// tensor-core path (fot_tc.cu)
-bool tc_supported(int rows, int cols);
-int tc_create(fot_ctx* c);
-void tc_destroy(fot_ctx* c);
-void half_step_tc(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
-                  float* pot_out, float* logsum);
-int64_t tc_terms(fot_ctx* c);
-void tc_begin(fot_ctx* c);
+                    float* pot_out, float* logsum);
+size_t tilt_bytes();
+cudaError_t plan_configure();
+int default_wait_limit();
 }  // namespace fot
 
 using namespace fot;
@@ -161,27 +156,33 @@ fot_status fot_create(fot_ctx** out, int rows, int cols, int precision, int devi
   for (float** b : bufs) ok = ok && cudaMalloc((void**)b, N * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->col_phi, (size_t)rows * sizeof(float)) == cudaSuccess;
   // the per-(16-output tile, row) plan of the larger banded pass (3 words each; rows padded to
-  // a multiple of 128, the plan's tile-major stride)
-  const size_t pr = (size_t)(rows + 127) / 128 * 128, pc = (size_t)(cols + 127) / 128 * 128;
+  // a multiple of 8, the plan's tile-major stride)
+  const size_t pr = (size_t)(rows + 7) / 8 * 8, pc = (size_t)(cols + 7) / 8 * 8;
   const size_t plan_words = 3 * std::max(pr * ((cols + 15) / 16), pc * ((rows + 15) / 16));
   ok = ok && cudaMalloc((void**)&c->plan, plan_words * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->red, (size_t)(4 * c->red_blocks + 16) * sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->err, sizeof(int)) == cudaSuccess;
-  ok = ok && cudaMalloc((void**)&c->terms, 2 * sizeof(unsigned long long)) == cudaSuccess;
-  if (ok) ok = cudaMemsetAsync(c->terms, 0, 2 * sizeof(unsigned long long), c->stream) == cudaSuccess;
+  const size_t term_bytes = (size_t)kTermSlots * 4 * sizeof(unsigned long long);
+  ok = ok && cudaMalloc((void**)&c->terms, term_bytes) == cudaSuccess;
+  if (ok) ok = cudaMemsetAsync(c->terms, 0, term_bytes, c->stream) == cudaSuccess;
   if (ok) ok = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) == cudaSuccess;
   if (ok) ok = cudaEventCreate(&c->ev_loop0) == cudaSuccess && cudaEventCreate(&c->ev_loop1) == cudaSuccess;
-  if (ok && simt_configure() != cudaSuccess) {   // per-device kernel attributes
+  if (ok && (simt_configure() != cudaSuccess || plan_configure() != cudaSuccess)) {   // per-device kernel attributes
     cudaGetLastError();
     fot_destroy(c);
     return FOT_ECUDA;
   }
-  if (ok && (precision == FOT_MIXED || precision == FOT_BF16)) {
-    if (!tc_supported(rows, cols)) {
-      fot_destroy(c);
-      return FOT_EUNSUPPORTED;
-    }
-    ok = tc_create(c) == 0;
+  if (precision == FOT_MIXED || precision == FOT_BF16)
+    ok = ok && cudaMalloc((void**)&c->tilt, tilt_bytes()) == cudaSuccess;
+  // items of the window kernel: groups of 8 rows x 4 tiles of at least 16
+  const size_t n_items = std::max(pr / 8 * ((cols + 63) / 64), pc / 8 * ((rows + 63) / 64));
+  ok = ok && cudaMalloc((void**)&c->items, n_items * sizeof(int4)) == cudaSuccess;
+  ok = ok && cudaMalloc((void**)&c->order, 2 * sizeof(int)) == cudaSuccess;
+  if (ok) ok = cudaMemsetAsync(c->order, 0, 2 * sizeof(int), c->stream) == cudaSuccess;
+  c->spin = default_wait_limit();
+  if (const char* e = getenv("FOT_TEST_WAIT_LIMIT")) {   // test-only: a short wait limit
+    const int v = atoi(e);
+    if (v > 0) c->spin = v;
   }
   if (!ok) {
     cudaGetLastError();
@@ -196,7 +197,9 @@ void fot_destroy(fot_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->device);
   cudaStreamSynchronize(c->stream);
-  if (c->tc) tc_destroy(c);
+  if (c->tilt) cudaFree(c->tilt);
+  if (c->items) cudaFree(c->items);
+  if (c->order) cudaFree(c->order);
   ktimer_free(c);
   if (c->loop_exec) cudaGraphExecDestroy(c->loop_exec);
   if (c->cap) cudaStreamDestroy(c->cap);
@@ -215,6 +218,7 @@ void fot_destroy(fot_ctx* c) {
 
 fot_status fot_set_stream(fot_ctx* c, void* s) {
   if (!c) return FOT_EINVAL;
+  if (c->stream != (cudaStream_t)s) tilt_reset(c);   // tables are rewritten on the new stream
   c->stream = (cudaStream_t)s;
   return FOT_OK;
 }
@@ -235,12 +239,14 @@ fot_status fot_work_count(fot_ctx* c, int64_t* terms_out, int64_t* tensor_terms_
 fot_status fot_work_split(fot_ctx* c, int64_t* out4) {
   if (!c || !out4) return FOT_EINVAL;
   FOT_CUDA(cudaSetDevice(c->device));
-  unsigned long long t[2] = {0, 0};
+  unsigned long long t[kTermSlots][4];
   FOT_CUDA(cudaMemcpyAsync(t, c->terms, sizeof(t), cudaMemcpyDeviceToHost, c->stream));
   FOT_CUDA(cudaStreamSynchronize(c->stream));
-  out4[0] = (int64_t)t[0];
-  out4[1] = (int64_t)t[1];
-  out4[2] = c->tc ? tc_terms(c) : 0;
+  for (int k = 0; k < 3; ++k) {
+    unsigned long long v = 0;
+    for (int i = 0; i < kTermSlots; ++i) v += t[i][k];
+    out4[k] = (int64_t)v;
+  }
   out4[3] = c->host_terms;
   return FOT_OK;
 }
@@ -311,19 +317,18 @@ fot_status fot_set_problem(fot_ctx* c, const float* g, const float* G) {
 
 static void half_step(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
                       float* pot_out, float* logsum) {
-  if ((c->precision == FOT_MIXED || c->precision == FOT_BF16) && c->tc)
-    half_step_tc(c, pot_in, lmarg, eps, pot_out, logsum);
-  else if (c->precision == FOT_FP32_DENSE)
+  if (c->precision == FOT_FP32_DENSE)
     half_step_simt(c, pot_in, lmarg, eps, pot_out, logsum, c->R);
   else
-    half_step_band(c, pot_in, lmarg, eps, pot_out, logsum, c->R);
+    half_step_band(c, pot_in, lmarg, eps, pot_out, logsum);
 }
 
 // the loop of Algorithm 1 for per-iteration eps e (px^2), enqueued on c->stream
 static void loop_body(fot_ctx* c, const std::vector<double>& e) {
   const int iters = (int)e.size();
-  if (c->tc) tc_begin(c);
   for (int t = 0; t < iters; ++t) {
+    // the tilt tables of the coming iterations, as many as the context holds
+    if (t % kTiltTables == 0) tilt_prepare(c, e.data() + t, std::min(iters - t, kTiltTables), &c->launches);
     // Eq. 7: f = eps (log a - log(Lambda V Lambda)); keep S of the last u-update (Eqs. 9-10)
     half_step(c, c->psi, c->la, e[(size_t)t], c->f, t == iters - 1 ? c->S_last : nullptr);
     // Eq. 8: psi = eps (log b - log(Lambda u Lambda))
@@ -378,8 +383,7 @@ static fot_status run_iterations(fot_ctx* c, const double* eps, int n_eps, int u
     if (cudaGraphLaunch(c->loop_exec, c->stream) != cudaSuccess) return FOT_ECUDA;
     cudaEventRecord(c->ev_loop1, c->stream);
     c->launches += c->loop_kernels;
-    // the host no longer knows which B table the device holds: the next pass rewrites it
-    if (c->tc) tc_begin(c);
+    tilt_reset(c);                         // (the tables now hold what the graph last wrote)
   } else {
     g_ktimer = c->ktimer;                  // null unless kernel timing is on
     cudaEventRecord(c->ev_loop0, c->stream);
@@ -645,7 +649,6 @@ fot_status fot_u_update(fot_ctx* c, const float* psi_in, double eps, float* f_ou
   if (!c || bad_ptr(psi_in) || bad_ptr(f_out) || !(eps > 0.0) || !isfinite(eps)) return FOT_EINVAL;
   if (!c->have_problem) return FOT_ESTATE;
   FOT_CUDA(cudaSetDevice(c->device));
-  if (c->tc) tc_begin(c);
   half_step(c, psi_in, c->la, eps, f_out, logsum_out);
   return check_launch(c);
 }
@@ -655,7 +658,6 @@ fot_status fot_v_update(fot_ctx* c, const float* f_in, double eps, float* psi_ou
   if (!c || bad_ptr(f_in) || bad_ptr(psi_out) || !(eps > 0.0) || !isfinite(eps)) return FOT_EINVAL;
   if (!c->have_problem) return FOT_ESTATE;
   FOT_CUDA(cudaSetDevice(c->device));
-  if (c->tc) tc_begin(c);
   half_step(c, f_in, c->lb, eps, psi_out, logsum_out);
   return check_launch(c);
 }

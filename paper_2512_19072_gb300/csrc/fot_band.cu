@@ -1,374 +1,314 @@
 // Banded axis passes: the same contraction as the exact pass,
 //     y[o][r] = log2 sum_m 2^( x[r][m]*scale - (o - m)^2 c ),   c = log2(e) / (2 eps),
-// but each output only visits the terms that can matter, and for large eps the inner loop
-// is a plain FP32 multiply-add GEMM instead of one exponential per term.
+// but each output only visits the terms that can matter, and where eps allows the inner sum is
+// a matrix product instead of one exponential per term.  A pass is two kernels: the window plan
+// (this file) and the window sums (fot_window.cuh, which describes the arithmetic).
 //
-// Work unit: one warp, 16 input rows r x one tile of 16 consecutive outputs o = k0 + i; lane
-// (h, i) = (lane / 16, lane % 16) owns rows 8h .. 8h+7 and output i.  Steps 1-2 run in
-// band_plan_kernel (one warp per row) and leave (alpha, lo, window length) per (row, tile);
-// steps 3-4 run in band_pass_kernel.
+// The plan leaves, per (row, tile of tile_w outputs), an offset alpha, the position mh it was
+// taken at and a window [lo, lo + wl):
 //
-// 1. Offset at every tile centre kc = k0 + 8: alpha_r, the largest term
-//    e_r(m, kc) = x_r[m] - (kc - m)^2 c over the positions that can hold the maximum, and the
-//    position where it is reached; within kPlanSlack below the exact maximum (see
-//    band_plan_kernel).
-// 2. A provable window: every o in the tile has max_m e_r(m, o) >= LB_r, with LB_r the
-//    value of that position's term at the worse tile end.  A 32-wide chunk of m whose
-//    upper bound (chunk maximum of x, nearest distance) over the whole tile is below
-//    LB_r - 40 holds only terms below 2^-40 of every output of the tile; the window is the
-//    hull of the remaining chunks (relative truncation error < len * 2^-40).
-// 3. Tilt identity (large eps).  With o = kc + kap:
-//      e_r(m, o) = [x_r[m] - (kc - m)^2 c - alpha_r] + [2 kap (m - Mref_r) c - kap^2 c]
-//                  + alpha_r + 2 kap (Mref_r - kc) c,
-//    so  sum_m 2^e = 2^(alpha_r + 2 kap (Mref_r - kc) c) * sum_m' A[r][m'] B[m'][kap]
-//    with A[r][m'] = 2^(e_r(lo_r + m', kc) - alpha_r) <= 2^kPlanSlack (one exponential per row and
-//    window position, shared by the tile's outputs) and B[m'][kap] = 2^(2 kap (m' - W/2) c -
-//    kap^2 c), the same for every row once each row's window is indexed from its own start
-//    lo_r (Mref_r = lo_r + W/2).  This is a GEMM over the window, done with FFMAs; the
-//    per-row offsets are the "online softmax" max-offsets of the paper's Toeplitz
-//    contraction (Sec. 3.1).  It is used when |B| stays within 2^+-40 and kap^2 c <= 32.
-// 4. Otherwise (small eps: narrow kernel, narrow windows) each output takes its exact
-//    maximum and sum over the window only.
-#include "fot_band_item.cuh"
+// 1. alpha = e(mh, kc), e(m, o) = x[m] scale - (o - m)^2 c, at the tile centre kc: the maximum
+//    over the 32-wide chunk whose own maximum gives the best term there.  It may lie below the
+//    exact maximum, which only raises the operands 2^(e - alpha) of the window sums (a sum that
+//    leaves the range of FP32 is done again there).
+// 2. A provable window: every o in the tile has max_m e(m, o) >= LB = min over the tile's two
+//    ends of e(mh, o) (e(mh, .) is concave).  A block of 8 positions whose bound (its maximum
+//    at its nearest distance to the tile) lies below LB - kCut holds only terms below 2^-kCut
+//    of every output of the tile; the window is the hull of the remaining blocks (found per
+//    32-wide chunk first, then narrowed from both ends).
+// 3. Whether the row's operands stay in range for the tilted product (row_in_range).
+// Arg-maxima carry the index in the low mantissa bits of the value they compare (5 bits for a
+// position, 7 for a chunk): one maximum instead of a compare and two selects; a chunk's maximum
+// is rounded by 2^-18 of itself that way, far inside the margin of kCut.
+//
+// What bounds it: latency and issue slots (4 MB of input at 1024^2, in L2).  Two lanes serve a
+// (row, tile): each takes every other pair of chunks (packed FP32 pairs), half of the scanned
+// chunk and one end of the window.  Chunks are padded to 36 words: lanes on different chunks read
+// different banks, lanes on the same chunk broadcast.
+#include "fot_window.cuh"
+
+#include <math.h>
 
 #include <algorithm>
 
 namespace fot {
 
-// Per (row, tile) plan (tiles of tile_w = 16, 32 or 64 outputs): offset alpha, window start
-// lo and window length wl.  A CTA takes R whole rows; each row is staged once in shared memory
-// as z[m] = x[m] * scale in 32-wide chunks (one pad word per chunk), with each chunk's maximum
-// cm[j] and the position p[j] where it is reached.  Then four lanes (q = 0..3) work on each
-// tile, eight tiles per warp, splitting the chunks (j = q mod 4) and the positions of a
-// scanned chunk (8 each) between them:
-//   a. alpha: the largest term e(m, kc) = z[m] - (kc - m)^2 c at the tile centre kc over the
-//      positions of the chunks scanned: first the chunk whose own maximum gives the best
-//      term at kc (e(p[j], kc)), then every chunk whose bound cm[j] - d_j^2 c (d_j its
-//      nearest distance to kc) exceeds the best term found so far by more than kPlanSlack,
-//      lowest first.  Every unscanned chunk is then within kPlanSlack of alpha, so
-//          alpha_exact - kPlanSlack <= alpha <= alpha_exact.
-//      An offset below the exact maximum only raises the operands 2^(e - alpha) (by at most
-//      2^kPlanSlack): the range arguments of the GEMM paths only need alpha <= alpha_exact.
-//   b. the window of step 2 above, with the lower bound LB = min over the tile ends o of
-//      e(mh, o) for the position mh that gave alpha (valid for every output of the tile, as
-//      e(mh, o) is concave in o): the first and the last chunk whose bound over the tile
-//      reaches LB - kCut.
-// With unit extents requested (tensor-core passes) the CTA also reduces, per tile, the union
-// of its rows' windows into the unit's [ext_lo, ext_hi) (all R rows lie in one 128-row block).
-constexpr int kPlanWarps = 8;                 // rows per CTA at most (plan rows are padded to a multiple)
-constexpr int kPlanMaxChunks = 4096 / kCW;    // 32-wide chunks of the longest row
-constexpr int kPlanQ = 4;                     // lanes per tile
-constexpr int kPlanTPW = 32 / kPlanQ;         // tiles per warp
-constexpr float kPlanSlack = 14.f;            // log2 units (a looser offset scans fewer chunks; the
-                                              // window test stays provable for any slack)
+namespace {
 
-// shared memory of one row (floats): z[n_chunks * 33], cm[n_chunks], p[n_chunks] (as float)
-__host__ __device__ inline int plan_row_floats(int n_chunks) { return n_chunks * (kCW + 3); }
+constexpr int kPlanRows = 8;                  // rows of a CTA: one row group of the window kernel
+constexpr int kPlanThreads = 512;
+constexpr int kPlanQ = 2;                     // lanes per (row, tile)
+constexpr int kZS = kCW + 4;                  // words of a staged chunk
 
-// max with the smaller key on ties, over the kPlanQ lanes of a tile
-__device__ __forceinline__ void quad_argmax(float& v, int& k) {
-#pragma unroll
-  for (int d = 1; d < kPlanQ; d <<= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, v, d);
-    const int ok = __shfl_xor_sync(0xffffffffu, k, d);
-    if (ov > v || (ov == v && ok < k)) {
-      v = ov;
-      k = ok;
-    }
-  }
+// shared memory of one row (floats): chunk maxima and minus their positions (rounded up to four
+// chunks each), block maxima [n_chunks * 4], z [n_chunks * kZS]
+__host__ __device__ inline int plan_row_floats(int n_chunks) { return 2 * ((n_chunks + 3) & ~3) + n_chunks * (4 + kZS); }
+
+// v with its low mantissa bits replaced by an index (-inf becomes a NaN, which fmaxf drops)
+template <int BITS>
+__device__ __forceinline__ float tagged(float v, int index) {
+  return __uint_as_float((__float_as_uint(v) & ~((1u << BITS) - 1u)) | (uint32_t)index);
 }
+template <int BITS>
+__device__ __forceinline__ int tag_of(float v) { return (int)(__float_as_uint(v) & ((1u << BITS) - 1u)); }
 
 template <int MAXP>
-__global__ void __launch_bounds__(1024) band_plan_kernel(const __grid_constant__ BandTable<MAXP> tab) {
+__global__ void __launch_bounds__(kPlanThreads) band_plan_kernel(const __grid_constant__ BandTable<MAXP> tab) {
   extern __shared__ __align__(16) float s_plan[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int wpr = tab.plan_wpr;                           // warps per row
-  const int R = (blockDim.x >> 5) / wpr;                  // rows of this CTA
-  const int rr = warp / wpr, wr = warp % wpr;             // this warp's row and tile group
-  // every row of a CTA belongs to one problem and one 128-row block: each problem's plan rows
-  // start at a multiple of 8 and R divides 8
-  const int grow0 = (int)blockIdx.x * R;
-  const BandArgs& a = tab.p[find_prob<MAXP, 1>(tab, grow0)];
-  const int row = grow0 + rr - a.plan_base;               // may be a padding row (>= n_rows)
+  const int tid = threadIdx.x;
+  const BandArgs& a = tab.p[find_prob<MAXP, 0>(tab, (int)blockIdx.x)];
+  const int rg = (int)blockIdx.x - a.plan_base;           // row group of the problem
   const int T = a.n_tiles, len = a.len, nch = a.n_chunks, tw = a.tile_w;
-  const bool live = row < a.n_rows && !error_latched(a.err);
-  const bool ext = a.ext_lo != nullptr;
-  float* z = s_plan + (size_t)rr * tab.plan_row_stride;
-  float* cm = z + nch * (kCW + 1);
-  float* cp = cm + nch;
-  int* s_ulo = reinterpret_cast<int*>(s_plan + (size_t)R * tab.plan_row_stride);
-  int* s_uhi = s_ulo + tab.plan_tiles;
-  if (a.ext_lo_next) {
-    // reset the next pass's unit extents (the problem's plan rows take strided shares; the
-    // next pass's plan kernel reduces into them): the whole array, since the next pass may
-    // contract the other axis with another tile width
-    if (wr == 0)
-      for (int i = row * 32 + lane; i < a.ext_units; i += a.plan_rows * 32) {
-        a.ext_lo_next[i] = 0x7F7F7F7F;
-        a.ext_hi_next[i] = 0;
-      }
-  }
-  if (ext)
-    for (int t = tid; t < T; t += blockDim.x) {
-      s_ulo[t] = 0x7F7F7F7F;
-      s_uhi[t] = 0;
-    }
   const float c = a.c, sc = a.x_scale;
-  // stage the rows (each warp of a row loads every wpr-th chunk, coalesced, eight in flight)
-  if (live) {
+  // threads per row: a power of two (at least kPlanQ lanes of one warp serve a (row, tile))
+  const int tpr = 1 << tab.plan_tpr_log2, rr = tid >> tab.plan_tpr_log2, ti = tid & (tpr - 1);
+  const int row = kPlanRows * rg + rr;
+  const bool live = row < a.n_rows;
+  float* const cm = s_plan + (size_t)rr * tab.plan_row_floats;
+  const int nchp = (nch + 3) & ~3;
+  float* const np_ = cm + nchp;                           // minus the maxima's positions
+  float* const bm = np_ + nchp;
+  float* const z = bm + 4 * nch;
+  // per item (four tiles): the span of its windows
+  int* const s_lo = reinterpret_cast<int*>(s_plan + (size_t)kPlanRows * tab.plan_row_floats);
+  int* const s_hi = s_lo + tab.plan_items;
+  for (int i = tid; i < a.items_row; i += blockDim.x) {
+    s_lo[i] = 0x7fffffff;
+    s_hi[i] = 0;
+  }
+  grid_wait();
+  grid_launch_next();
+
+  // ---- stage: blocks of 8 positions, a thread each; four neighbouring threads share a chunk
+  {
     const float* xr = a.x + (size_t)row * len;
-    for (int j0 = wr; j0 < nch; j0 += 8 * wpr) {
+    const bool vec = (a.vec & 1) != 0;
+    const f32x2 sc2 = pack2(sc, sc);
+    for (int b = ti; b < nchp * 4; b += tpr) {
+      const int m0 = b * 8, j = b >> 2, u0 = (b & 3) * 8;
       float v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int j = j0 + q * wpr, m = j * kCW + lane;
-        v[q] = (j < nch && m < len) ? __fmul_rn(__ldg(xr + m), sc) : -INFINITY;
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int j = j0 + q * wpr;
-        if (j < nch) z[j * (kCW + 1) + lane] = v[q];
-      }
-    }
-  }
-  __syncthreads();
-  // chunk maxima and their leftmost positions (thread per chunk; the pad word puts the lanes
-  // of a warp on different banks)
-  if (live) {
-    for (int j = wr * 32 + lane; j < nch; j += wpr * 32) {
-      const float* zj = z + j * (kCW + 1);
-      float best = -INFINITY;
-      int arg = 0;
-#pragma unroll 8
-      for (int u = 0; u < kCW; ++u) {
-        const float v = zj[u];
-        if (v > best) {
-          best = v;
-          arg = u;
-        }
-      }
-      cm[j] = best;
-      cp[j] = (float)(j * kCW + arg);
-    }
-  }
-  __syncthreads();
-
-  if (live) {
-    const size_t np = (size_t)a.plan_stride * T;
-    float* p_alpha = a.plan;
-    int* p_lo = reinterpret_cast<int*>(a.plan + np);
-    int* p_wl = reinterpret_cast<int*>(a.plan + 2 * np);
-    const int q = lane & (kPlanQ - 1);
-    // warp-uniform loop over this warp's groups of eight tiles (the combines and the candidate
-    // rounds below are warp-wide); lanes of a missing tile compute nothing and write nothing
-    for (int tg = wr * kPlanTPW; tg < T; tg += wpr * kPlanTPW) {
-      const int t = tg + lane / kPlanQ;
-      const bool has = t < T;
-      const int k0 = min(t, T - 1) * tw, kc = k0 + tw / 2, k1 = min(k0 + tw, len) - 1;
-      const float fkc = (float)kc;
-      auto bound = [&](int j) {                           // chunk j's bound at kc
-        const int clo = j * kCW, chi = min(clo + kCW, len) - 1;
-        const int dd = clo > kc ? clo - kc : (chi < kc ? kc - chi : 0);
-        return fmaf(-(float)dd * (float)dd, c, cm[j]);
-      };
-      // a. the chunk whose maximum gives the best term at kc
-      float vb = -INFINITY;
-      int jb = 0x7fffffff;
-      for (int j = q; j < nch && has; j += kPlanQ) {
-        const float d = fkc - cp[j];
-        const float v = fmaf(-d * d, c, cm[j]);
-        if (v > vb) {
-          vb = v;
-          jb = j;
-        }
-      }
-      quad_argmax(vb, jb);
-      float alpha = -INFINITY;
-      int mh = 0x7fffffff;
-      // exact maximum over chunk j, the four lanes taking eight positions each; every lane of
-      // the warp runs it (the combine is warp-wide), a lane whose tile has nothing to scan
-      // passes valid = false and keeps its maximum
-      auto scan = [&](int j, bool valid) {
-        const float* zj = z + j * (kCW + 1) + q * (kCW / kPlanQ);
-        float d = fkc - (float)(j * kCW + q * (kCW / kPlanQ));
-        float v0 = -INFINITY;
-        int m0 = 0x7fffffff;
-#pragma unroll
-        for (int u = 0; u < kCW / kPlanQ; ++u, d -= 1.f) {
-          const float v = fmaf(-d * d, c, zj[u]);
-          if (v > v0) {
-            v0 = v;
-            m0 = j * kCW + q * (kCW / kPlanQ) + u;
-          }
-        }
-        quad_argmax(v0, m0);
-        if (valid && (v0 > alpha || (v0 == alpha && m0 < mh))) {
-          alpha = v0;
-          mh = m0;
-        }
-      };
-      const bool any = has && vb != -INFINITY;
-      if (__any_sync(0xffffffffu, any)) {
-        scan(any ? jb : 0, any);
-        // the candidate chunks (this lane's share), then rounds in which every tile scans its
-        // lowest remaining candidate together; each is tested again against the maximum so far
-        uint32_t cand[kPlanMaxChunks / 32 / kPlanQ + 1];
-#pragma unroll
-        for (int w = 0; w < kPlanMaxChunks / 32 / kPlanQ + 1; ++w) cand[w] = 0u;
-        if (any)
-          for (int j = q, b = 0; j < nch; j += kPlanQ, ++b)
-            if (j != jb && bound(j) > alpha + kPlanSlack) cand[b >> 5] |= 1u << (b & 31);
-        for (;;) {
-          int mine = 0x7fffffff;                          // this lane's lowest candidate chunk
-#pragma unroll
-          for (int w = 0; w < kPlanMaxChunks / 32 / kPlanQ + 1; ++w)
-            if (mine == 0x7fffffff && cand[w] != 0u) mine = (w * 32 + __ffs(cand[w]) - 1) * kPlanQ + q;
-          float dummy = 0.f;
-          int next = mine;
-          quad_argmax(dummy, next);                       // the tile's lowest candidate
-          if (!__any_sync(0xffffffffu, next != 0x7fffffff)) break;
-          if (next != 0x7fffffff && next == mine) {
-            const int b = (mine - q) / kPlanQ;
-            cand[b >> 5] &= ~(1u << (b & 31));
-          }
-          const bool doscan = next != 0x7fffffff && bound(next) > alpha + kPlanSlack;
-          scan(doscan ? next : 0, doscan);
-        }
-      }
-      // b. window
-      int wlo = 0x7fffffff, whi = -1;
-      if (has && alpha != -INFINITY) {
-        const float zm = z[(mh / kCW) * (kCW + 1) + mh % kCW];
-        const float da = (float)(k0 - mh), db = (float)(k1 - mh);
-        const float lb = fminf(fmaf(-da * da, c, zm), fmaf(-db * db, c, zm));
-        for (int j = q; j < nch; j += kPlanQ) {
-          const int clo = j * kCW, chi = min(clo + kCW, len) - 1;
-          const int d = clo > k1 ? clo - k1 : (chi < k0 ? k0 - chi : 0);
-          if (fmaf(-(float)d * (float)d, c, cm[j]) >= lb - kCut) {
-            wlo = min(wlo, j);
-            whi = max(whi, j);
-          }
-        }
-      }
-#pragma unroll
-      for (int d = 1; d < kPlanQ; d <<= 1) {
-        wlo = min(wlo, __shfl_xor_sync(0xffffffffu, wlo, d));
-        whi = max(whi, __shfl_xor_sync(0xffffffffu, whi, d));
-      }
-      if (!has || q != 0) continue;
-      const size_t pi = (size_t)t * a.plan_stride + row;
-      if (alpha == -INFINITY) {                           // no finite term: empty row
-        p_alpha[pi] = -INFINITY;
-        p_lo[pi] = 0;
-        p_wl[pi] = 0;
+      if (live && vec && m0 + 8 <= len) {
+        const float4 p = __ldg(reinterpret_cast<const float4*>(xr + m0)), q = __ldg(reinterpret_cast<const float4*>(xr + m0) + 1);
+        v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
+        v[4] = q.x; v[5] = q.y; v[6] = q.z; v[7] = q.w;
       } else {
-        const int lo = wlo * kCW, hi = min((whi + 1) * kCW, len);
-        p_alpha[pi] = alpha;
-        p_lo[pi] = lo;
-        p_wl[pi] = hi - lo;
-        if (ext) {
-          atomicMin(&s_ulo[t], lo);
-          atomicMax(&s_uhi[t], hi);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = live && m0 + u < len ? __ldg(xr + m0 + u) : -INFINITY;
+      }
+      float best = -INFINITY, top = -INFINITY;            // block maximum; the same with its position
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        unpack2(mul2(pack2(v[u], v[u + 1]), sc2), v[u], v[u + 1]);
+        best = fmaxf(best, fmaxf(v[u], v[u + 1]));
+        top = fmaxf(top, fmaxf(tagged<5>(v[u], u0 + u), tagged<5>(v[u + 1], u0 + u + 1)));
+      }
+      if (j < nch) {
+        float4* const zb = reinterpret_cast<float4*>(z + j * kZS + u0);
+        zb[0] = make_float4(v[0], v[1], v[2], v[3]);
+        zb[1] = make_float4(v[4], v[5], v[6], v[7]);
+        bm[b] = best;
+      }
+      // (the four threads of a chunk are neighbours and take this iteration together)
+      const unsigned quad = 0xfu << (tid & 28);
+      top = fmaxf(top, __shfl_xor_sync(quad, top, 1));
+      top = fmaxf(top, __shfl_xor_sync(quad, top, 2));
+      best = fmaxf(best, __shfl_xor_sync(quad, best, 1));
+      best = fmaxf(best, __shfl_xor_sync(quad, best, 2));
+      if (u0 == 0) {
+        cm[j] = best;
+        np_[j] = -(float)(j * kCW + tag_of<5>(top));
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- kPlanQ lanes per (row, tile)
+  const size_t np = (size_t)a.plan_stride * T;
+  int* const plan_i = reinterpret_cast<int*>(a.plan);
+  const int q = ti & (kPlanQ - 1);
+  const float kmax = 0.5f * (float)tw;
+  const f32x2 nc2 = pack2(-c, -c);
+  // (lanes past the tiles or rows compute on a valid place and write nothing: the shuffles below
+  // want whole warps)
+  for (int t0 = 0; t0 < T; t0 += tpr / kPlanQ) {
+    const int t = min(t0 + ti / kPlanQ, T - 1);
+    const bool has = live && t0 + ti / kPlanQ < T;
+    const float f0 = (float)(t * tw) + a.shift;            // the tile's ends and centre
+    const float f1 = (float)(min((t + 1) * tw, a.n_out) - 1) + a.shift;
+    const float fkc = (float)(t * tw + tw / 2) + a.shift;
+
+    // the chunk whose maximum gives the best term at kc
+    float vb = -INFINITY;
+    const f32x2 kc2 = pack2(fkc, fkc);
+#pragma unroll 4
+    for (int j = 2 * q; j < nchp; j += 2 * kPlanQ) {
+      const float2 m = *reinterpret_cast<const float2*>(cm + j), p = *reinterpret_cast<const float2*>(np_ + j);
+      const f32x2 d = add2(kc2, pack2(p.x, p.y));
+      float v0, v1;
+      unpack2(fma2(mul2(d, d), nc2, pack2(m.x, m.y)), v0, v1);
+      vb = fmaxf(vb, fmaxf(tagged<7>(v0, j), tagged<7>(v1, j + 1)));
+    }
+#pragma unroll
+    for (int d = 1; d < kPlanQ; d <<= 1) vb = fmaxf(vb, __shfl_xor_sync(0xffffffffu, vb, d));
+    const bool any = vb != -INFINITY;                     // some term is finite
+    const int jb = any ? tag_of<7>(vb) : 0;
+
+    // the maximum over that chunk (half of it for each lane)
+    float sb = -INFINITY;
+    {
+      constexpr int kShare = kCW / kPlanQ;
+      const float* zj = z + jb * kZS + q * kShare;
+      const float d0 = fkc - (float)(jb * kCW + q * kShare);
+      f32x2 d01 = pack2(d0, d0 - 1.f);
+      const f32x2 dn2 = pack2(-2.f, -2.f);
+#pragma unroll
+      for (int u = 0; u < kShare; u += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(zj + u);
+        float v0, v1, v2, v3;
+        unpack2(fma2(mul2(d01, d01), nc2, pack2(x.x, x.y)), v0, v1);
+        d01 = add2(d01, dn2);
+        unpack2(fma2(mul2(d01, d01), nc2, pack2(x.z, x.w)), v2, v3);
+        d01 = add2(d01, dn2);
+        const int i = q * kShare + u;
+        sb = fmaxf(sb, fmaxf(tagged<5>(v0, i), tagged<5>(v1, i + 1)));
+        sb = fmaxf(sb, fmaxf(tagged<5>(v2, i + 2), tagged<5>(v3, i + 3)));
+      }
+    }
+#pragma unroll
+    for (int d = 1; d < kPlanQ; d <<= 1) sb = fmaxf(sb, __shfl_xor_sync(0xffffffffu, sb, d));
+    const int ub = tag_of<5>(sb);
+    const float zm = z[jb * kZS + ub];
+    int mh = jb * kCW + ub;
+    const float fm = (float)mh;
+    const float dk = fkc - fm, da = f0 - fm, db = f1 - fm;
+    const float alpha = fmaf(-dk * dk, c, zm);
+    const float lb = fminf(fmaf(-da * da, c, zm), fmaf(-db * db, c, zm)) - kCut;
+
+    // the window in chunks
+    int wlo = 0x7fffffff, whi = -1;
+    {
+      const float c0 = (float)(2 * q * kCW);
+      f32x2 e0 = pack2(f0 - c0 - (float)(kCW - 1), f0 - c0 - (float)(2 * kCW - 1));   // f0 - chunk's last
+      f32x2 e1 = pack2(c0 - f1, c0 + (float)kCW - f1);                                // chunk's first - f1
+      const f32x2 up = pack2((float)(2 * kPlanQ * kCW), (float)(2 * kPlanQ * kCW));
+      const f32x2 dn = pack2(-(float)(2 * kPlanQ * kCW), -(float)(2 * kPlanQ * kCW));
+#pragma unroll 4
+      for (int j = 2 * q; j < nchp; j += 2 * kPlanQ) {
+        const float2 m = *reinterpret_cast<const float2*>(cm + j);
+        float a0, a1, b0, b1, v0, v1;
+        unpack2(e0, a0, a1);
+        unpack2(e1, b0, b1);
+        const f32x2 d = pack2(fmaxf(fmaxf(a0, b0), 0.f), fmaxf(fmaxf(a1, b1), 0.f));
+        e0 = add2(e0, dn);
+        e1 = add2(e1, up);
+        unpack2(fma2(mul2(d, d), nc2, pack2(m.x, m.y)), v0, v1);
+        if (v0 >= lb) {
+          wlo = min(wlo, j);
+          whi = j;
+        }
+        if (v1 >= lb) {
+          wlo = min(wlo, j + 1);
+          whi = j + 1;
         }
       }
     }
-  }
-  if (ext) {
-    // the CTA's rows share one row block: one global atomic pair per tile
-    __syncthreads();
-    const int rb = (grow0 - a.plan_base) / 128;
-    for (int t = tid; t < T; t += blockDim.x) {
-      if (s_uhi[t] > 0) {
-        atomicMin(&a.ext_lo[rb * T + t], s_ulo[t]);
-        atomicMax(&a.ext_hi[rb * T + t], s_uhi[t]);
+#pragma unroll
+    for (int d = 1; d < kPlanQ; d <<= 1) {
+      wlo = min(wlo, __shfl_xor_sync(0xffffffffu, wlo, d));
+      whi = max(whi, __shfl_xor_sync(0xffffffffu, whi, d));
+    }
+    // narrow the hull block by block, chunk by chunk: lane 0 from its start, lane 1 from its end
+    // (it holds mh's block, whose bound reaches LB)
+    const bool win = any && whi >= 0;
+    int j = win ? (q == 0 ? wlo : whi) : 0, edge = 0;
+    const int jend = win ? (q == 0 ? whi : wlo) : 0, jstep = q == 0 ? 1 : -1;
+    for (;;) {
+      const float4 m = *reinterpret_cast<const float4*>(bm + 4 * j);
+      const float ms[4] = {m.x, m.y, m.z, m.w};
+      const float a0 = f0 - (float)(j * kCW) - 7.f, b0 = (float)(j * kCW) - f1;
+      int mask = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float d = fmaxf(fmaxf(a0 - 8.f * i, b0 + 8.f * i), 0.f);
+        if (fmaf(-d * d, c, ms[i]) >= lb) mask |= 1 << i;
+      }
+      edge = 4 * j + (q == 0 ? (mask ? __ffs(mask) - 1 : 0) : (mask ? 32 - __clz(mask) : 4));
+      if (mask != 0 || j == jend) break;
+      j += jstep;
+    }
+    const int other = __shfl_xor_sync(0xffffffffu, edge, 1);
+    if (has && q == 0) {
+      const int lo = win ? edge * 8 : 0, hi = win ? min(other * 8, len) : 0;
+      mh = max(lo, min(mh, hi - 1));
+      const bool in = !win || row_in_range(kmax, lo, hi, mh, c);
+      const size_t pi = (size_t)t * a.plan_stride + row;
+      a.plan[pi] = any ? alpha : -INFINITY;
+      plan_i[np + pi] = lo | ((hi - lo) << 16);
+      plan_i[2 * np + pi] = mh | (in ? 0 : 1 << 16);
+      if (hi > lo) {
+        atomicMin(&s_lo[t / kWinWarps], lo);
+        atomicMax(&s_hi[t / kWinWarps], hi);
       }
     }
   }
+  if (a.group != kPlanRows) return;                       // exact windows only: no item list
+  __syncthreads();
+  // the items of this row group: those with a wide span to the front of the list
+  for (int i = tid; i < a.items_row; i += blockDim.x) {
+    const int lo = s_hi[i] > 0 ? s_lo[i] : 0, hi = s_hi[i];
+    const bool wide = hi - lo > a.wide_span;
+    const int at = wide ? atomicAdd(&a.order[0], 1) : a.n_items - 1 - atomicAdd(&a.order[1], 1);
+    a.items[at] = make_int4(rg, i, lo, hi);
+  }
 }
 
-#ifndef FOT_BAND_MIN_BLOCKS
-#define FOT_BAND_MIN_BLOCKS 2   // resident CTAs per SM the register budget is sized for (at 3
-                                // the 80-register budget spills; measured slower)
-#endif
-
-template <int MODE, int MAXP>
-__global__ void __launch_bounds__(kBW * 32, FOT_BAND_MIN_BLOCKS) band_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
-  __shared__ __align__(16) float sA[kBW][2 * kSA];
-  const int warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * kBW + warp;
-  if (gw >= tab.items) return;                            // warp-uniform
-  const BandArgs& a = tab.p[find_prob<MAXP, 2>(tab, gw)];
-  if (error_latched(a.err)) return;
-  const int lw = gw - a.item_base;
-  const int tile = lw % a.n_tiles, r0 = (lw / a.n_tiles) * 2 * kBR;
-  // each item takes exactly one of the two (warp-uniform choice inside band_item)
-  band_item<MODE, 0>(a, r0, tile, tile * kBT, sA[warp]);
-  band_item<MODE, 1>(a, r0, tile, tile * kBT, sA[warp]);
-}
-
+// finish a table: chunk and tile counts, prefix sums
 template <int MAXP>
-void band_table_finish(BandTable<MAXP>& t) {
-  int rows = 0, plans = 0, items = 0, ctas = 0, tiles = 1;
+void finish(BandTable<MAXP>& t, int* max_chunks) {
+  int plans = 0, items = 0, pitch = 16, chunks = 1, items_row = 1;
   for (int q = 0; q < t.n; ++q) {
     BandArgs& a = t.p[q];
     a.n_chunks = (a.len + kCW - 1) / kCW;
-    a.n_tiles = (a.len + a.tile_w - 1) / a.tile_w;
-    a.plan_stride = (a.n_rows + 127) / 128 * 128;
-    a.plan_rows = (a.n_rows + kPlanWarps - 1) / kPlanWarps * kPlanWarps;
-    a.row_base = rows;
+    a.n_tiles = (a.n_out + a.tile_w - 1) / a.tile_w;
+    a.plan_stride = (a.n_rows + 7) / 8 * 8;
+    a.items_row = (a.n_tiles + kWinWarps - 1) / kWinWarps;
+    a.vec = 0;
+    if ((a.len & 3) == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0) a.vec |= 1;
+    const uintptr_t outs = reinterpret_cast<uintptr_t>(a.y) | reinterpret_cast<uintptr_t>(a.lmarg) |
+                           reinterpret_cast<uintptr_t>(a.logsum);
+    if ((a.n_rows & 1) == 0 && (outs & 7u) == 0) a.vec |= 2;
     a.plan_base = plans;
     a.item_base = items;
-    a.cta_base = ctas;
-    rows += a.n_rows;
-    plans += a.plan_rows;
-    items += ((a.n_rows + 2 * kBR - 1) / (2 * kBR)) * a.n_tiles;
-    ctas += ((a.n_rows + 127) / 128) * a.n_tiles;
-    tiles = std::max(tiles, a.n_tiles);
+    plans += (a.n_rows + kPlanRows - 1) / kPlanRows;
+    a.n_items = (a.n_rows + a.group - 1) / a.group * a.items_row;
+    items += a.n_items;
+    items_row = std::max(items_row, a.items_row);
+    chunks = std::max(chunks, a.n_chunks);
+    pitch = std::max(pitch, stage_pitch(a.len));
   }
-  t.rows = rows;
   t.plans = plans;
   t.items = items;
-  t.ctas = ctas;
-  t.plan_tiles = tiles;
+  t.plan_items = items_row;
+  t.pitch_max = std::min(pitch, kPitchCap);
+  t.plan_row_floats = plan_row_floats(chunks);
+  *max_chunks = chunks;
 }
 
-template <int MAXP>
-void band_prepare(cudaStream_t s, BandTable<MAXP>& t) {
-  int nch = 1;
-  for (int q = 0; q < t.n; ++q) nch = std::max(nch, t.p[q].n_chunks);
-  t.plan_row_stride = plan_row_floats(nch);
-  // warps per row: enough tile groups of eight for the widest row of tiles (at most 32); rows
-  // per CTA: a power of two up to 8 (a CTA never straddles two problems or two 128-row
-  // blocks) within 8 warps per CTA (or the row's own warps) and the default 48 KB of shared
-  // memory together with the per-tile unit extents
-  int wpr = std::max(1, std::min(32, (t.plan_tiles + kPlanTPW - 1) / kPlanTPW));
-  t.plan_wpr = wpr;
-  const size_t tile_bytes = 2 * sizeof(int) * (size_t)t.plan_tiles;
-  int R = 8;
-  while (R > 1 && (R * wpr > std::max(8, wpr) || R * t.plan_row_stride * sizeof(float) + tile_bytes > 48 * 1024)) R /= 2;
-  const size_t smem = (size_t)R * t.plan_row_stride * sizeof(float) + tile_bytes;
-  ktimer_begin(s, kKPlan);
-  band_plan_kernel<MAXP><<<t.plans / R, R * wpr * 32, smem, s>>>(t);
-  ktimer_end(s);
+}  // namespace
+
+// Tile width for a problem with kernel constant c.  A row's operands stay in range while
+// tile_w (D + mh - lo) c <= kRangeMax, D the farthest window position from mh.  For a smooth
+// potential the window W is about the tile plus the distance sqrt(kCut / c) on both sides at which
+// the Gaussian has fallen by 2^-kCut, with mh in its middle: tile_w W c.  The limit for 32 leaves
+// room for windows half as wide again (rows outside the bound cost more there).  The wider tile
+// shares each exponential, and each unit's set-up, between more outputs.
+int tile_width_for(float c) {
+  const float reach = 2.f * sqrtf(kCut / c);
+  if (32.f * (32.f + reach) * c <= 70.f) return 32;
+  if (16.f * (16.f + reach) * c <= 100.f) return 16;
+  return 0;
 }
 
-template <int MODE, int MAXP>
-void band_simt(cudaStream_t s, const BandTable<MAXP>& t) {
-  ktimer_begin(s, kKBand);
-  band_pass_kernel<MODE, MAXP><<<(t.items + kBW - 1) / kBW, kBW * 32, 0, s>>>(t);
-  ktimer_end(s);
-}
-
-template void band_table_finish<1>(BandTable<1>&);
-template void band_table_finish<kMaxBatch>(BandTable<kMaxBatch>&);
-template void band_prepare<1>(cudaStream_t, BandTable<1>&);
-template void band_prepare<kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&);
-template void band_simt<kBandLse, 1>(cudaStream_t, const BandTable<1>&);
-template void band_simt<kBandPot, 1>(cudaStream_t, const BandTable<1>&);
-template void band_simt<kBandLse, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
-template void band_simt<kBandPot, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
-
-// the two passes of one half-step for one context
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale) {
   BandArgs a{};
   a.x = x;
@@ -380,30 +320,144 @@ BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, 
   a.eps = (float)eps;
   a.n_rows = n_rows;
   a.len = len;
-  a.tile_w = kBT;
+  a.n_out = len;
+  const int tw = tile_width_for(a.c);
+  a.tile_w = tw == 0 ? 16 : tw;
+  a.group = tw == 0 ? 2 : 8;
+  a.items = c->items;
+  a.order = c->order;
+  a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
+  if (tw != 0)
+    for (int i = 0; i < 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
   return a;
 }
 
+template <int MODE, int MAXP>
+void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
+  int chunks = 1;
+  finish(t, &chunks);
+  // plan: threads per row to the next power of two of the widest row's (tile, lane) pairs
+  int tiles = 1;
+  for (int q = 0; q < t.n; ++q) tiles = std::max(tiles, t.p[q].n_tiles);
+  int tl = 2;                                             // (four threads stage a chunk together)
+  while ((1 << tl) < tiles * kPlanQ && (kPlanRows << tl) < kPlanThreads) ++tl;
+  t.plan_tpr_log2 = tl;
+  const size_t plan_smem = (size_t)kPlanRows * t.plan_row_floats * sizeof(float) + 2 * t.plan_items * sizeof(int);
+  ktimer_begin(s, kKPlan);
+  launch_dependent(band_plan_kernel<MAXP>, dim3(t.plans), kPlanRows << tl, plan_smem, s, t);
+  ktimer_end(s);
+  ktimer_begin(s, form == kFormFp32 ? kKBand : kKTensor);
+  if (form == kFormFp32)
+    window_launch<MODE, kFormFp32, MAXP>(s, t);
+  else if (form == kFormSplit)
+    window_launch<MODE, kFormSplit, MAXP>(s, t);
+  else
+    window_launch<MODE, kFormSingle, MAXP>(s, t);
+  ktimer_end(s);
+}
+
+template void band_pass<0, 1>(cudaStream_t, BandTable<1>&, int);
+template void band_pass<1, 1>(cudaStream_t, BandTable<1>&, int);
+template void band_pass<0, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
+template void band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
+
+// the plan kernel stages eight rows: more than the default 48 KB from rows of 1152 on
+cudaError_t plan_configure() {
+  const int lim = (int)(kPlanRows * plan_row_floats(4096 / kCW) * sizeof(float)) + 2 * 64 * (int)sizeof(int);
+  cudaError_t e = cudaFuncSetAttribute(band_plan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(band_plan_kernel<kMaxBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  return e;
+}
+
+int default_wait_limit() { return kSpinDefault; }
+
+int form_of(const fot_ctx* c) {
+  return c->precision == FOT_MIXED ? kFormSplit : c->precision == FOT_BF16 ? kFormSingle : kFormFp32;
+}
+
+// ---- tilt tables of the BF16 forms ---------------------------------------------------------
+
+namespace {
+
+struct TiltArgs {
+  uint4* out;
+  int tw[kTiltTables / 4];                    // four 8-bit tile widths per word
+  float c[kTiltTables];
+};
+
+// One table: fragments of T[kap][p] = 2^(2 kap p c), kap = row - tw/2, split into BF16 hi and lo
+// parts in the register order of mma.m16n8k16's A operand, with the columns permuted as the
+// window kernel produces them (lane q of a quad owns positions 4q .. 4q + 3).
+__global__ void tilt_table_kernel(const __grid_constant__ TiltArgs t) {
+  const int i = blockIdx.x, mt = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tw = (t.tw[i >> 2] >> (8 * (i & 3))) & 255;
+  if (16 * mt >= tw) return;
+  uint32_t hi[4], lo[4];
+  tilt_fragments_bf16(t.c[i], 16 * mt - tw / 2, lane, hi, lo);
+  uint4* o = t.out + (size_t)i * kTiltWords + (size_t)mt * 64 + lane;
+  o[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  o[32] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+}  // namespace
+
+size_t tilt_bytes() { return (size_t)kTiltTables * kTiltWords * sizeof(uint4); }
+
+void tilt_reset(fot_ctx* c) { c->tilt_eps.clear(); }
+
+void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
+  if (!c->tilt) return;
+  TiltArgs t{};
+  t.out = c->tilt;
+  c->tilt_eps.clear();
+  for (int i = 0; i < n && (int)c->tilt_eps.size() < kTiltTables; ++i) {
+    if (!c->tilt_eps.empty() && c->tilt_eps.back() == eps[i]) continue;
+    const float cc = (float)(1.4426950408889634 / (2.0 * eps[i]));
+    const int tw = tile_width_for(cc);
+    if (tw == 0) continue;                    // exact windows only: no table
+    const int k = (int)c->tilt_eps.size();
+    t.c[k] = cc;
+    t.tw[k >> 2] |= tw << (8 * (k & 3));
+    c->tilt_eps.push_back(eps[i]);
+  }
+  if (c->tilt_eps.empty()) return;
+  ktimer_begin(c->stream, kKPlan);            // timed with the plans (set-up of the passes)
+  tilt_table_kernel<<<(unsigned)c->tilt_eps.size(), 64, 0, c->stream>>>(t);
+  ktimer_end(c->stream);
+  ++*launches;
+}
+
+const uint4* tilt_for(fot_ctx* c, double eps, int tile_w, int64_t* launches) {
+  if (!c->tilt || tile_w == 0) return nullptr;
+  for (size_t i = 0; i < c->tilt_eps.size(); ++i)
+    if (c->tilt_eps[i] == eps) return c->tilt + i * kTiltWords;
+  tilt_prepare(c, &eps, 1, launches);
+  return c->tilt;
+}
+
 // One half-step with banded passes: pot_out = eps (lmarg - log(Lambda exp(pot_in/eps) Lambda)).
-void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
-                    float* pot_out, float* logsum, float* tmp) {
+void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double eps, float* pot_out,
+                    float* logsum) {
+  const int form = form_of(c);
   BandTable<1> t{};
   t.n = 1;
+  t.spin_limit = c->spin;
+  int64_t k = 2 * 2;
   // pass over the contiguous axis: rows of pot_in, outputs along cols, written [k][L]
   t.p[0] = band_args(c, pot_in, c->rows, c->cols, eps, (float)(1.4426950408889634 / eps));
-  t.p[0].y = tmp;
-  band_table_finish(t);
-  band_prepare(c->stream, t);
-  band_simt<kBandLse>(c->stream, t);
-  // pass over the row axis (input tmp[k][L], log2 units) with the fused potential update
-  t.p[0] = band_args(c, tmp, c->cols, c->rows, eps, 1.f);
+  t.p[0].y = c->R;
+  const uint4* tilt = tilt_for(c, eps, t.p[0].group == 8 ? t.p[0].tile_w : 0, &k);
+  t.p[0].tilt = tilt;
+  band_pass<0>(c->stream, t, form);
+  // pass over the row axis (input R[k][L], log2 units) with the fused potential update
+  t.p[0] = band_args(c, c->R, c->cols, c->rows, eps, 1.f);
+  t.p[0].tilt = tilt;
   t.p[0].y = pot_out;
   t.p[0].lmarg = lmarg;
   t.p[0].logsum = logsum;
-  band_table_finish(t);
-  band_prepare(c->stream, t);
-  band_simt<kBandPot>(c->stream, t);
-  c->launches += 4;
+  band_pass<1>(c->stream, t, form);
+  c->launches += k;
 }
 
 }  // namespace fot

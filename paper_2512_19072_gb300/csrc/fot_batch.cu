@@ -2,9 +2,8 @@
 // stream of multi-problem launches.
 //
 // Every axis pass of every problem goes into the same two launches (the window plan, then the
-// banded window sums on the CUDA cores or, for the mixed form, on the tensor cores):
-// the kernels take a table of up to 64 problems by value and map each warp / CTA to its
-// problem by prefix sums (BandTable).  The whole solve - problem setup and all iterations
+// window sums), whatever tile width each problem takes: the kernels take a table of up to 64
+// problems by value and map each CTA to its problem by prefix sums (BandTable).  The whole solve - problem setup and all iterations
 // with each iteration's eps baked into its launches - is captured once into a CUDA graph and
 // replayed with a single cudaGraphLaunch; the graph is rebuilt only when the inputs, the
 // schedule or the iteration count change.
@@ -14,7 +13,7 @@
 #include <math.h>
 #include <string.h>
 
-#include <chrono>
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -22,8 +21,6 @@
 
 namespace fot {
 void set_problem_simt(fot_ctx* c, const float* g, const float* G, float* psi0, float psi0_val);
-BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale);
-int tc_create(fot_ctx* c);
 }  // namespace fot
 
 using namespace fot;
@@ -55,56 +52,39 @@ static void capture_solve(fot_batch* b, cudaStream_t st, const float* const* g, 
     set_problem_simt(c, g[q], G[q], c->psi, psi0);
     k += 3;
   }
-  // one table per pass and tile width: a problem runs the same kernels as its single solve
-  static const int kWidths[4] = {64, 32, 16, 0};
+  const int form = use_tc ? kFormSplit : kFormFp32;
   BandTable<kMaxBatch>* tab = new BandTable<kMaxBatch>();
-  std::vector<BandArgs> p1(n), p2(n);
-  std::vector<int> width(n);
-  std::vector<fot_ctx*> tctx(n);
-  if (use_tc)
-    for (fot_ctx* c : b->ctx) tc_begin(c);
+  tab->n = n;
+  tab->spin_limit = b->ctx[0]->spin;
+  std::vector<double> sched((size_t)iters);
+  std::vector<BandArgs> p2((size_t)n);
   for (int it = 0; it < iters; ++it) {
+    if (use_tc && it % kTiltTables == 0)
+      for (int q = 0; q < n; ++q) {
+        // the problem's tilt tables of the coming iterations
+        const int m = std::min(iters - it, kTiltTables);
+        for (int t = 0; t < m; ++t) sched[(size_t)t] = eps[(size_t)q * n_eps + (n_eps == 1 ? 0 : it + t)];
+        tilt_prepare(b->ctx[q], sched.data(), m, &k);
+      }
     for (int half = 0; half < 2; ++half) {
       for (int q = 0; q < n; ++q) {
         fot_ctx* c = b->ctx[q];
         const double e = eps[(size_t)q * n_eps + (n_eps == 1 ? 0 : it)];
-        const float* pin = half == 0 ? c->psi : c->f;
-        float* pout = half == 0 ? c->f : c->psi;
-        BandArgs a1 = band_args(c, pin, c->rows, c->cols, e, (float)(1.4426950408889634 / e));
+        BandArgs& a1 = tab->p[q];
+        a1 = band_args(c, half == 0 ? c->psi : c->f, c->rows, c->cols, e, (float)(1.4426950408889634 / e));
         a1.y = c->R;
-        BandArgs a2 = band_args(c, c->R, c->cols, c->rows, e, 1.f);
-        a2.y = pout;
+        if (use_tc) a1.tilt = tilt_for(c, e, a1.group == 8 ? a1.tile_w : 0, &k);
+        BandArgs& a2 = p2[(size_t)q];
+        a2 = band_args(c, c->R, c->cols, c->rows, e, 1.f);
+        a2.y = half == 0 ? c->f : c->psi;
         a2.lmarg = half == 0 ? c->la : c->lb;
         a2.logsum = (half == 0 && it == iters - 1) ? c->S_last : nullptr;
-        p1[q] = a1;
-        p2[q] = a2;
-        width[q] = use_tc ? tc_width_for(a1.c) : -1;
+        a2.tilt = a1.tilt;
       }
-      for (int pass = 0; pass < 2; ++pass) {
-        const std::vector<BandArgs>& pa = pass == 0 ? p1 : p2;
-        for (int wi = 0; wi < (use_tc ? 4 : 1); ++wi) {
-          tab->n = 0;
-          for (int q = 0; q < n; ++q)
-            if (width[q] == (use_tc ? kWidths[wi] : -1)) {
-              tctx[tab->n] = b->ctx[q];
-              tab->p[tab->n++] = pa[q];
-            }
-          if (tab->n == 0) continue;
-          if (use_tc) {
-            for (int j = 0; j < tab->n; ++j) tc_bind(tctx[j], tab->p[j]);
-            k += pass == 0 ? tc_pass<0>(st, *tab, kWidths[wi], tctx.data())
-                           : tc_pass<1>(st, *tab, kWidths[wi], tctx.data());
-          } else {
-            band_table_finish(*tab);
-            band_prepare(st, *tab);
-            if (pass == 0)
-              band_simt<0>(st, *tab);
-            else
-              band_simt<1>(st, *tab);
-            k += 2;
-          }
-        }
-      }
+      band_pass<0>(st, *tab, form);
+      std::copy(p2.begin(), p2.end(), tab->p);
+      band_pass<1>(st, *tab, form);
+      k += 4;
     }
   }
   delete tab;
@@ -238,6 +218,7 @@ fot_status fot_batch_solve(fot_batch* b, const float* const* g, const float* con
     b->key_neps = n_eps;
   }
   if (cudaGraphLaunch(b->exec, b->stream) != cudaSuccess) return FOT_ECUDA;
+  for (fot_ctx* c : b->ctx) tilt_reset(c);   // (the tables hold what the graph last wrote)
   for (fot_ctx* c : b->ctx) {
     c->have_problem = true;
     c->have_solution = true;

@@ -41,9 +41,9 @@ __device__ __forceinline__ bool error_latched(const int* err) {
 // context with timing on runs its loop, g_ktimer points at its timer and every launch site
 // brackets its kernel with a pair of events; fot_kernel_times sums them per class.
 enum KernelClass : int {
-  kKPlan = FOT_KERNEL_PLAN,       // band_plan_kernel
-  kKBand = FOT_KERNEL_BAND,       // band_pass_kernel
-  kKTensor = FOT_KERNEL_TENSOR,   // tc_pass_kernel
+  kKPlan = FOT_KERNEL_PLAN,       // band_plan_kernel and the tilt tables
+  kKBand = FOT_KERNEL_BAND,       // window_pass_kernel, FP32 form
+  kKTensor = FOT_KERNEL_TENSOR,   // window_pass_kernel, BF16 forms
   kKDense = FOT_KERNEL_DENSE,     // axis_pass_kernel (dense exact pass)
   kKClasses = FOT_KERNEL_CLASSES
 };
@@ -81,8 +81,8 @@ struct fot_ctx {
   double* red = nullptr;     // reduction scratch (partials + results)
   float* lam_hat = nullptr;  // cFOT: the spectra of lambda (allocated by the first cFOT solve)
   int* err = nullptr;        // latched device status
-  unsigned long long* terms = nullptr;  // device counters of evaluated (row, output, m) terms on
-                                        // the CUDA cores: [0] banded GEMM, [1] exact windows
+  unsigned long long* terms = nullptr;  // device counters of evaluated (row, output, m) terms
+                                        // (BandArgs::terms)
   int64_t host_terms = 0;    // terms of passes whose count is known on the host (dense)
   int red_blocks = 0;
   // host-side state
@@ -101,8 +101,12 @@ struct fot_ctx {
   cudaGraphExec_t loop_exec = nullptr;
   std::vector<double> loop_key;
   int64_t loop_kernels = 0;
-  // mixed-precision (tensor-core) resources, owned by fot_tc.cu
-  void* tc = nullptr;
+  // BF16 forms: tilt tables of the window sums (device) and the eps each was written for
+  uint4* tilt = nullptr;
+  std::vector<double> tilt_eps;
+  int spin = 0;              // polls of a bounded device wait
+  int4* items = nullptr;     // item list of the window kernel
+  int* order = nullptr;      // [2] its counters
   fot::KernelTimer* ktimer = nullptr;   // per-kernel-class loop timing, when switched on
 };
 

@@ -1,0 +1,17 @@
+// The window kernels (fot_window.cuh) of one operand form, in a translation unit of its own so
+// that the forms compile in parallel.
+#include "fot_window.cuh"
+
+namespace fot {
+
+template <int MODE, int FORM, int MAXP>
+void window_launch(cudaStream_t s, const BandTable<MAXP>& t) {
+  launch_dependent(window_pass_kernel<MODE, FORM, MAXP>, dim3(t.items), kWinThreads, window_smem(t.pitch_max), s, t);
+}
+
+template void window_launch<0, kFormSingle, 1>(cudaStream_t, const BandTable<1>&);
+template void window_launch<1, kFormSingle, 1>(cudaStream_t, const BandTable<1>&);
+template void window_launch<0, kFormSingle, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
+template void window_launch<1, kFormSingle, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
+
+}  // namespace fot

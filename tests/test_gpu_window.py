@@ -1,0 +1,66 @@
+"""The window sums of the banded passes at the edges of their units: half-steps against the FP64
+oracle where tiles, row groups and windows end raggedly, where an item's rows do not fit its
+staging buffer, where 32-wide units have to be cut or summed exactly, and where a potential's
+steps put the plan's offsets far below the exact maxima.
+
+Tolerances as in test_gpu_parity: FP32 rounding of the potentials (POT_RTOL), plus 2^-15 eps for
+the split-BF16 form (two passes, each product within 2^-16)."""
+import numpy as np
+import pytest
+
+from oracle import fot
+from paper_2512_19072_gb300 import inputs
+from fot_testutil import POT_RTOL, f32, to_dev, to_np
+
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:invalid value encountered")]
+
+
+def _check(B, prec, psi, eps, seed):
+    shape = psi.shape
+    rng = np.random.default_rng(seed)
+    g = f32(rng.uniform(0.05, 1.0, size=shape))
+    G = f32(rng.uniform(0.05, 1.0, size=shape))
+    g[rng.uniform(size=shape) < 0.1] = 0.0
+    g[-1, -1] = 0.5
+    ctx = B.fot_create(*shape, {"fp32": B.FOT_FP32, "mixed": B.FOT_MIXED}[prec])
+    B.fot_set_problem(ctx, to_dev(g), to_dev(G))
+    f = to_np(B.fot_u_update(ctx, to_dev(psi), eps))
+    B.fot_sync(ctx)
+    ctx.close()
+    ref, _ = fot.u_update(psi, fot.log0(fot.marginal(g)), eps)
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isneginf(f), np.isneginf(ref))
+    tol = POT_RTOL * np.abs(ref[fin]).max() + (2.0 ** -15 * eps if prec == "mixed" else 0.0)
+    err = np.abs(f[fin] - ref[fin]).max()
+    assert err <= tol, (err, tol)
+
+
+# rows and columns around multiples of the row group (8), the tiles (16, 32) and the four tiles of
+# an item, aligned and unaligned; eps for exact windows, 16-wide and 32-wide units
+@pytest.mark.parametrize("prec", ["fp32", "mixed"])
+@pytest.mark.parametrize("shape", [(7, 129), (9, 127), (33, 64), (65, 66), (24, 1)])
+@pytest.mark.parametrize("eps", [1.5, 20.0, 400.0])
+def test_ragged_units(fot_lib, prec, shape, eps):
+    psi = f32(inputs.random_potential(*shape, scale=0.3 * max(shape) ** 2 + 3 * eps, seed=5, zero_frac=0.15))
+    _check(fot_lib, prec, psi, eps, 1)
+
+
+# windows over whole rows of 1500 and 1499: more than an item's staging buffer holds
+@pytest.mark.parametrize("prec", ["fp32", "mixed"])
+@pytest.mark.parametrize("shape", [(10, 1500), (10, 1499)])
+def test_rows_beyond_the_staging_buffer(fot_lib, prec, shape):
+    psi = f32(inputs.random_potential(*shape, scale=2e4, seed=6))
+    _check(fot_lib, prec, psi, 1e5, 2)
+
+
+# two far-apart plateaus of equal height: the maximum jumps across the row within a tile, so the
+# window spans the gap and the operands leave the tilted product's range
+@pytest.mark.parametrize("prec", ["fp32", "mixed"])
+@pytest.mark.parametrize("n,eps", [(640, 100.0), (641, 60.0), (640, 8.0)])
+def test_windows_across_a_gap(fot_lib, prec, n, eps):
+    k = np.arange(n, dtype=np.float64)
+    row = np.full(n, -np.inf)
+    row[:24] = 0.5 * (n / 2 - k[:24]) ** 2                 # the two ends tie at the centre
+    row[-24:] = 0.5 * (n / 2 - k[-24:]) ** 2
+    psi = np.stack([row + 0.3 * eps * i for i in range(12)])
+    _check(fot_lib, prec, f32(psi), eps, 3)
