@@ -339,8 +339,8 @@ fot_status fot_work_count(fot_ctx* ctx, int64_t* terms_out, int64_t* tensor_term
 
 /* The same count split by how the terms were evaluated: out4[0] banded products of FP32
  * operands, out4[1] banded exact windows (one exponential per term), out4[2] banded products of
- * BF16 operands, out4[3] dense exact passes (including the phase step's moment passes).
- * Synchronising.  The paper has no counterpart: a measurement aid. */
+ * BF16 operands, out4[3] dense exact passes.  (The phase step's moment passes count with the
+ * first two, or with the dense ones in a FOT_FP32_DENSE context.)  Synchronising.  The paper has no counterpart: a measurement aid. */
 fot_status fot_work_split(fot_ctx* ctx, int64_t* out4);
 
 /* Kernel classes of fot_kernel_times. */

@@ -29,7 +29,7 @@
 namespace fot {
 void half_step_dispatch(fot_ctx* c, const float* pot_in, const float* lmarg, double eps, float* pot_out,
                         float* logsum);
-void moments_simt(fot_ctx* c, const float* psi, const float* S, double eps, double dx, float* Dx, float* Dy);
+void moments(fot_ctx* c, const float* psi, const float* S, double eps, double dx, float* Dx, float* Dy);
 void set_problem_simt(fot_ctx* c, const float* g, const float* G, float* psi0, float psi0_val);
 void fill(fot_ctx* c, float* p, size_t N, float v);
 }  // namespace fot
@@ -268,7 +268,7 @@ extern "C" fot_status fot_backward(fot_ctx* c, const float* g, const float* G, c
     trapezoid_vjp_col<<<1, 1, 0, s>>>(colb, c->rows, c->cols, (float)c->dx, Dxb);
     float* Dx = Lp;
     float* Dy = Ln;
-    moments_simt(c, psi_cur, c->S_last, eT, c->dx, Dx, Dy);
+    moments(c, psi_cur, c->S_last, eT, c->dx, Dx, Dy);
     moments_vjp_pre<<<gN, 256, 0, s>>>(Dxb, Dyb, Dx, Dy, (float)(1.0 / eT), N, fb, ab);
     // K(Dxbar e^{-S}), K(Dybar e^{-S}) on the target grid (4 log-domain applications)
     split_kernel<<<gN, 256, 0, s>>>(Dxb, c->S_last, (float)eT, N, pp, pn);

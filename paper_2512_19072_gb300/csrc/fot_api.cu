@@ -17,6 +17,7 @@ void half_step_simt(fot_ctx* c, const float* pot_in, const float* lmarg, double 
 cudaError_t simt_configure();
 void moments_simt(fot_ctx* c, const float* psi, const float* S, double eps, double dx,
                   float* Dx, float* Dy);
+void moments_band(fot_ctx* c, const float* psi, const float* S, double eps, double dx, float* Dx, float* Dy);
 void set_problem_simt(fot_ctx* c, const float* g, const float* G, float* psi0, float psi0_val);
 void fill(fot_ctx* c, float* p, size_t N, float v);
 void source_stats(fot_ctx* c, const float* f, const float* S, double eps, double* out);
@@ -34,6 +35,16 @@ void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double 
 size_t tilt_bytes();
 cudaError_t plan_configure();
 int default_wait_limit();
+}  // namespace fot
+
+namespace fot {
+// the phase step's moments in the context's way: every term, or banded
+void moments(fot_ctx* c, const float* psi, const float* S, double eps, double dx, float* Dx, float* Dy) {
+  if (c->precision == FOT_FP32_DENSE)
+    moments_simt(c, psi, S, eps, dx, Dx, Dy);
+  else
+    moments_band(c, psi, S, eps, dx, Dx, Dy);
+}
 }  // namespace fot
 
 using namespace fot;
@@ -583,7 +594,7 @@ fot_status fot_phase(fot_ctx* c, float* phi_out, float* dphidx_out, float* dphid
   FOT_CUDA(cudaSetDevice(c->device));
   float* Dx = dphidx_out ? dphidx_out : c->tmp;
   float* Dy = dphidy_out ? dphidy_out : c->tmp2;
-  moments_simt(c, c->psi, c->S_last, c->eps_last, c->dx, Dx, Dy);
+  moments(c, c->psi, c->S_last, c->eps_last, c->dx, Dx, Dy);
   if (phi_out) integrate_phase(c, Dx, Dy, c->dx, phi_out);
   fot_status s = check_launch(c);
   if (s != FOT_OK) return s;
@@ -599,7 +610,7 @@ fot_status fot_moments(fot_ctx* c, const float* psi, const float* logsum_u, doub
   const double h = dx > 0.0 ? dx : 1.0 / sqrt(n);
   float* Dx = dphidx_out ? dphidx_out : c->tmp;
   float* Dy = dphidy_out ? dphidy_out : c->tmp2;
-  moments_simt(c, psi, logsum_u, eps, h, Dx, Dy);
+  moments(c, psi, logsum_u, eps, h, Dx, Dy);
   if (phi_out) integrate_phase(c, Dx, Dy, h, phi_out);
   fot_status s = check_launch(c);
   if (s != FOT_OK) return s;
@@ -680,7 +691,7 @@ fot_status fot_solve_phase_host(fot_ctx* c, const float* g_host, const float* G_
   FOT_CUDA(cudaMemcpyAsync(c->tmp2, G_host, bytes, cudaMemcpyHostToDevice, c->stream));
   fot_status s = fot_solve(c, c->tmp, c->tmp2, dx, eps, n_eps, eps_units, iters);
   if (s != FOT_OK) return s;
-  moments_simt(c, c->psi, c->S_last, c->eps_last, c->dx, c->tmp, c->tmp2);
+  moments(c, c->psi, c->S_last, c->eps_last, c->dx, c->tmp, c->tmp2);
   integrate_phase(c, c->tmp, c->tmp2, c->dx, c->phi);
   s = check_launch(c);
   if (s != FOT_OK) return s;

@@ -332,8 +332,8 @@ BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, 
   return a;
 }
 
-template <int MODE, int MAXP>
-void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
+template <int MAXP>
+void plan_pass(cudaStream_t s, BandTable<MAXP>& t) {
   int chunks = 1;
   finish(t, &chunks);
   // plan: threads per row to the next power of two of the widest row's (tile, lane) pairs
@@ -346,6 +346,14 @@ void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
   ktimer_begin(s, kKPlan);
   launch_dependent(band_plan_kernel<MAXP>, dim3(t.plans), kPlanRows << tl, plan_smem, s, t);
   ktimer_end(s);
+}
+
+template void plan_pass<1>(cudaStream_t, BandTable<1>&);
+template void plan_pass<kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&);
+
+template <int MODE, int MAXP>
+void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
+  plan_pass(s, t);
   ktimer_begin(s, form == kFormFp32 ? kKBand : kKTensor);
   if (form == kFormFp32)
     window_launch<MODE, kFormFp32, MAXP>(s, t);

@@ -29,6 +29,12 @@ struct BandArgs {
                        // rows they read (written by the plan)
   int* order;          // [2] items placed at the front and at the back so far
   const uint4* tilt;           // BF16 forms: operand fragments of the tilt matrix for (c, tile_w)
+  // moment passes only (fot_moments.cu): term weights, a second output, the logarithm of the
+  // divisor, and the coordinate of index m, coord0 + m coord_step
+  const float* w;      // [n_rows][len]
+  float* y2;           // layout of y
+  const float* off;    // natural log, layout of y
+  float coord0, coord_step;
   float x_scale, c, eps, shift;
   int n_rows, len, n_out;
   int tile_w;          // outputs per plan tile and window unit: 16 or 32
@@ -89,6 +95,10 @@ BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, 
 // log-sum output; MODE 1: potential update).  Two kernel launches.
 template <int MODE, int MAXP>
 void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form);
+
+// the window plan alone, for a table whose window kernel the caller launches (fot_moments.cu)
+template <int MAXP>
+void plan_pass(cudaStream_t s, BandTable<MAXP>& t);
 
 int form_of(const fot_ctx* c);
 

@@ -188,7 +188,8 @@ void half_step_simt(fot_ctx* c, const float* pot_in, const float* lmarg, double 
   launch_pass<8, kLsePot>(c, q);
 }
 
-// Phase-gradient moments (Eqs. 9-10, ratio form with u/g^2 = exp(-S_last)).
+// Phase-gradient moments (Eqs. 9-10, ratio form with u/g^2 = exp(-S_last)), every term (contexts of
+// FOT_FP32_DENSE; the others take moments_band).
 void moments_simt(fot_ctx* c, const float* psi, const float* S, double eps, double dx,
                   float* Dx, float* Dy) {
   const int rows = c->rows, cols = c->cols;

@@ -590,16 +590,23 @@ __device__ __noinline__ void other_unit(const BandArgs& a, int r0, int k0, RowVi
   }
 }
 
-template <int MODE, int FORM, int MAXP>
-__global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
-  extern __shared__ __align__(128) float s_x[];           // four -inf (padded to 64 bytes), then the rows
-  __shared__ __align__(8) uint64_t s_bar;
+// A warp's unit of the item that its CTA was launched for.
+struct Unit {
+  RowView rv;
+  int r0, k0, row;                                        // first row and output, this lane's row
+  bool pairs, out_of_range, skip;
+};
+
+// The start of a window CTA: read the item and this warp's plan entries, stage the rows; `meanwhile`
+// runs while they are on their way.  s_x: four -inf (padded to 64 bytes), then the rows.  False: the
+// warp has nothing to do.
+template <int MAXP, typename F>
+__device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const BandArgs& a, float* s_x, uint64_t* s_bar, Unit& u,
+                                          F meanwhile) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int prob = MAXP == 1 ? 0 : find_prob<MAXP, 1>(tab, (int)blockIdx.x);
-  const BandArgs& a = tab.p[prob];
-  const bool pairs = a.group == 2;
+  u.pairs = a.group == 2;
   if (tid == 0) {
-    mbar_init(smem_addr(&s_bar), 1);
+    mbar_init(smem_addr(s_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 4) s_x[tid] = -INFINITY;
@@ -607,10 +614,10 @@ __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window
   grid_wait();
   grid_launch_next();
   if (tid < 2 && (int)blockIdx.x == a.item_base) a.order[tid] = 0;   // for the next pass's plan
-  const bool skip = error_latched(a.err);                 // an error is latched: write nothing
+  u.skip = error_latched(a.err);                          // an error is latched: write nothing
   // the item: row group, four tiles, and the span of the rows that they read
   int rg, tg, base, top;
-  if (pairs) {
+  if (u.pairs) {
     const int local = (int)blockIdx.x - a.item_base;
     rg = local / a.items_row;
     tg = local - rg * a.items_row;
@@ -626,68 +633,85 @@ __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window
   const int r0 = a.group * rg;
   const int pitch = stage_pitch(top - base);
   const bool staged = top > base && pitch <= tab.pitch_max;
-  if (staged && (a.vec & 1) && warp == 0) {
+  const bool bulk = staged && (a.vec & 1);
+  const int nr = min(a.group, a.n_rows - r0);
+  if (bulk && warp == 0) {
     const uint32_t bytes = (uint32_t)(top - base) * 4u;   // the ends are multiples of 4 here
-    const int nr = min(a.group, a.n_rows - r0);
     __syncwarp();
-    if (lane == 0) mbar_expect(smem_addr(&s_bar), bytes * nr);
+    if (lane == 0) mbar_expect(smem_addr(s_bar), bytes * nr);
     __syncwarp();
     if (lane < nr)
-      bulk_load(smem_addr(rows + lane * pitch), a.x + (size_t)(r0 + lane) * a.len + base, bytes, smem_addr(&s_bar));
+      bulk_load(smem_addr(rows + lane * pitch), a.x + (size_t)(r0 + lane) * a.len + base, bytes, smem_addr(s_bar));
   }
   // the plan entry of this lane's row, for its warp's tile
-  const int tile = tg * kWinWarps + warp, k0 = tile * a.tile_w;
-  const int lr = pairs ? lane >> 4 : lane >> 2;
-  const int row = r0 + lr;
-  RowView rv;
+  const int tile = tg * kWinWarps + warp;
+  const int lr = u.pairs ? lane >> 4 : lane >> 2;
+  u.r0 = r0;
+  u.k0 = tile * a.tile_w;
+  u.row = r0 + lr;
+  RowView& rv = u.rv;
   rv.alpha = -INFINITY;
   int w1 = 0, w2 = 0;
-  if (tile < a.n_tiles && row < a.n_rows) {
-    const size_t np = (size_t)a.plan_stride * a.n_tiles, pi = (size_t)tile * a.plan_stride + row;
+  if (tile < a.n_tiles && u.row < a.n_rows) {
+    const size_t np = (size_t)a.plan_stride * a.n_tiles, pi = (size_t)tile * a.plan_stride + u.row;
     rv.alpha = a.plan[pi];
     w1 = reinterpret_cast<const int*>(a.plan)[np + pi];
     w2 = reinterpret_cast<const int*>(a.plan)[2 * np + pi];
   }
-  Tilt<FORM> tilt;
-  if (!pairs) tilt.load(a, a.tile_w, true);
+  meanwhile();
   rv.lo = w1 & 0xffff;
   rv.wl = w1 >> 16;
   rv.mh = w2 & 0xffff;
+  u.out_of_range = (w2 >> 16) != 0;
   rv.staged = staged;
   rv.vec = staged || (a.vec & 1);
-  rv.row = staged ? rows + lr * pitch - base : a.x + (size_t)min(row, a.n_rows - 1) * a.len;
+  rv.row = staged ? rows + lr * pitch - base : a.x + (size_t)min(u.row, a.n_rows - 1) * a.len;
   rv.saddr = smem_addr(rows + lr * pitch) - 4u * (uint32_t)base;
   rv.minf = smem_addr(s_x);
-  bool ok = true;
-  if (staged && !(a.vec & 1)) {
+  if (staged && !bulk) {
     // rows that are not 16-byte aligned: plain loads, -inf up to the next multiple of 4
-    const int n4 = (top - base + 3) & ~3, nr = min(a.group, a.n_rows - r0);
+    const int n4 = (top - base + 3) & ~3;
     const float* src = a.x + (size_t)r0 * a.len + base;
     for (int r = warp; r < nr; r += kWinWarps)
       for (int i = lane; i < n4; i += 32)
         rows[r * pitch + i] = base + i < a.len ? __ldg(src + (size_t)r * a.len + i) : -INFINITY;
   }
   __syncthreads();                                        // (the barrier's initialisation, the -inf, plain rows)
-  if (staged && (a.vec & 1)) ok = stage_wait(smem_addr(&s_bar), 0, tab.spin_limit, a.err);
-  if (!__all_sync(0xffffffffu, ok) || tile >= a.n_tiles) return;
+  const bool ok = !bulk || stage_wait(smem_addr(s_bar), 0, tab.spin_limit, a.err);
+  return __all_sync(0xffffffffu, ok) && tile < a.n_tiles;
+}
+
+template <int MODE, int FORM, int MAXP>
+__global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
+  extern __shared__ __align__(128) float s_x[];
+  __shared__ __align__(8) uint64_t s_bar;
+  const int lane = threadIdx.x & 31;
+  const BandArgs& a = tab.p[find_prob<MAXP, 1>(tab, (int)blockIdx.x)];
+  Unit u;
+  Tilt<FORM> tilt;
+  if (!open_unit(tab, a, s_x, &s_bar, u, [&]() {
+        if (a.group != 2) tilt.load(a, a.tile_w, true);
+      }))
+    return;
   unsigned long long* terms = a.terms + 4 * (blockIdx.x & (kTermSlots - 1));
-  if (pairs) {
+  const RowView& rv = u.rv;
+  if (u.pairs) {
     if ((lane & 15) == 0 && rv.wl > 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
-    exact_pair<MODE>(a, row, k0, rv.lo, rv.wl, rv.mh, rv.row, rv.vec, skip);
+    exact_pair<MODE>(a, u.row, u.k0, rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
     return;
   }
   const int W = __reduce_max_sync(0xffffffffu, rv.wl);
-  const bool in_range = !__any_sync(0xffffffffu, (w2 >> 16) != 0);
+  const bool in_range = !__any_sync(0xffffffffu, u.out_of_range);
   if (in_range && lane == 0 && W > 0)
     atomicAdd(terms + (FORM == kFormFp32 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
-  const bool here = in_range && (staged || W == 0);
+  const bool here = in_range && (rv.staged || W == 0);
   if (here) {
-    const float kc = (float)(k0 + (a.tile_w >> 1)) + a.shift;
-    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, r0, k0, kc, rv, W, tilt, skip)
-                       : gemm_unit<MODE, FORM, 16, true>(a, r0, k0, kc, rv, W, tilt, skip))
+    const float kc = (float)(u.k0 + (a.tile_w >> 1)) + a.shift;
+    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, tilt, u.skip)
+                       : gemm_unit<MODE, FORM, 16, true>(a, u.r0, u.k0, kc, rv, W, tilt, u.skip))
       return;
   }
-  other_unit<MODE, FORM>(a, r0, k0, rv, W, in_range && !here, skip, terms);
+  other_unit<MODE, FORM>(a, u.r0, u.k0, rv, W, in_range && !here, u.skip, terms);
 }
 
 // launch with programmatic dependence on the kernel before it in the stream: its set-up (and

@@ -64,3 +64,21 @@ def test_windows_across_a_gap(fot_lib, prec, n, eps):
     row[-24:] = 0.5 * (n / 2 - k[-24:]) ** 2
     psi = np.stack([row + 0.3 * eps * i for i in range(12)])
     _check(fot_lib, prec, f32(psi), eps, 3)
+
+
+# the moment passes at the same edges, against the oracle's moments; tolerance as in
+# test_moments_kernel_matches_oracle (FP32 rounding of the logarithms, times the largest coordinate)
+@pytest.mark.parametrize("shape,eps", [((7, 129), 1.5), ((33, 66), 20.0), ((65, 40), 300.0), ((10, 1499), 1e5)])
+def test_moments_at_unit_edges(fot_lib, shape, eps):
+    B = fot_lib
+    psi = f32(inputs.random_potential(*shape, scale=0.02 * max(shape) ** 2 + 3 * eps, seed=8, zero_frac=0.15))
+    S = f32(fot.log_kernel_apply(psi, eps) + np.random.default_rng(9).normal(0, 0.2, size=shape))
+    dx = 0.41
+    ctx = B.fot_create(*shape)
+    _, Dx, Dy = (to_np(t) for t in B.fot_moments(ctx, to_dev(psi), to_dev(S), eps, dx))
+    ctx.close()
+    Dx_r, Dy_r = fot.moments(psi, S, eps, dx)
+    lmax = (np.abs(S).max() + np.abs(psi[np.isfinite(psi)]).max() / eps) / np.log(2)
+    cmax = max(shape) / 2 / (min(shape) * dx)
+    tol = 4 * 2.0 ** -24 * lmax * cmax + 1e-6 * max(np.abs(Dx_r).max(), np.abs(Dy_r).max())
+    assert np.abs(Dx - Dx_r).max() <= tol and np.abs(Dy - Dy_r).max() <= tol
