@@ -151,13 +151,15 @@ fot_status fot_select_eps(fot_ctx* ctx, const float* g, const float* G, double d
  * is a rectangular rows_in x rows_out (cols_in x cols_out) matrix:
  *     f   = eps (log a - log(Lambda_r V Lambda_c^T))    on the input grid,
  *     psi = eps (log b - log(Lambda_r^T u Lambda_c))    on the output grid,
- * a = g^2/sum g^2, b = G^2/sum G^2, start V = 1/(rows_out cols_out).  Every axis pass is dense
- * and exact in FP32 (each output's own maximum, then the sum), as FOT_FP32_DENSE.
+ * a = g^2/sum g^2, b = G^2/sum G^2, start V = 1/(rows_out cols_out).  The axis passes
+ * are the banded FP32 passes of FOT_FP32 (they were dense and exact before: results agree to FP32
+ * rounding).
  *   g: rows_in x cols_in and G: rows_out x cols_out amplitudes, row-major FP32 device memory;
  *   eps in px^2 (n_eps == 1, or n_eps == iters for one value per iteration); f_out
  *   (rows_in x cols_in) and psi_out (rows_out x cols_out): device buffers of the caller that
  *   receive the potentials (px^2, -inf at zero mass); cuda_stream: the stream (NULL: default).
- * The call allocates and frees its temporaries (3 images and a few words) and synchronises the
+ * The call allocates and frees its temporaries (3 images, a window plan of 3 words per 16 pixels
+ * and a few words) and synchronises the
  * stream before returning.  Errors: FOT_EINVAL (a null pointer, a size < 1 or > 3072,
  * iters < 1, n_eps other than 1 or iters, eps not finite and > 0), FOT_EMASS (g or G without
  * mass), FOT_ENOMEM, FOT_ENONFINITE (a non-finite potential), FOT_ECUDA. */

@@ -309,26 +309,30 @@ int tile_width_for(float c) {
   return 0;
 }
 
+void band_set_eps(BandArgs& a, double eps) {
+  a.c = (float)(1.4426950408889634 / (2.0 * eps));
+  a.eps = (float)eps;
+  const int tw = tile_width_for(a.c);
+  a.tile_w = tw == 0 ? 16 : tw;
+  a.group = tw == 0 ? 2 : 8;
+  a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
+  if (tw != 0)
+    for (int i = 0; i < 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
+}
+
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale) {
   BandArgs a{};
   a.x = x;
   a.plan = c->plan;
   a.err = c->err;
   a.terms = c->terms;
+  a.items = c->items;
+  a.order = c->order;
   a.x_scale = x_scale;
-  a.c = (float)(1.4426950408889634 / (2.0 * eps));
-  a.eps = (float)eps;
   a.n_rows = n_rows;
   a.len = len;
   a.n_out = len;
-  const int tw = tile_width_for(a.c);
-  a.tile_w = tw == 0 ? 16 : tw;
-  a.group = tw == 0 ? 2 : 8;
-  a.items = c->items;
-  a.order = c->order;
-  a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
-  if (tw != 0)
-    for (int i = 0; i < 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
+  band_set_eps(a, eps);
   return a;
 }
 

@@ -88,6 +88,9 @@ __device__ __forceinline__ int find_prob(const BandTable<MAXP>& t, int gi) {
 // outputs).
 int tile_width_for(float c);
 
+// the fields of a pass that follow from eps: kernel constant, tile width, step scales
+void band_set_eps(BandArgs& a, double eps);
+
 // fill one pass's arguments; the tilt fragments and the outputs are set by the caller
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale);
 

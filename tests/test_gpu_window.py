@@ -82,3 +82,23 @@ def test_moments_at_unit_edges(fot_lib, shape, eps):
     cmax = max(shape) / 2 / (min(shape) * dx)
     tol = 4 * 2.0 ** -24 * lmax * cmax + 1e-6 * max(np.abs(Dx_r).max(), np.abs(Dy_r).max())
     assert np.abs(Dx - Dx_r).max() <= tol and np.abs(Dy - Dy_r).max() <= tol
+
+
+# unequal grids: half-integer shifts, an output axis longer or shorter than the input axis, exact
+# windows and 16- and 32-wide units; FP32 rounding of the potentials over the iterations
+@pytest.mark.parametrize("shape_in,shape_out,eps", [((40, 51), (57, 36), 2.0), ((33, 130), (96, 23), 25.0),
+                                                    ((70, 64), (64, 203), 500.0)])
+def test_unequal_grids_at_unit_edges(fot_lib, shape_in, shape_out, eps):
+    from oracle import rect
+    from fot_testutil import solve_rtol
+    rng = np.random.default_rng(12)
+    g = f32(rng.uniform(0.05, 1.0, size=shape_in))
+    G = f32(rng.uniform(0.05, 1.0, size=shape_out))
+    G[rng.uniform(size=shape_out) < 0.2] = 0.0
+    iters = 6
+    f, psi = (to_np(t) for t in fot_lib.fot_solve_rect(to_dev(g), to_dev(G), [eps], iters))
+    r = rect.fot_iterate_rect(g, G, eps, iters)
+    for got, ref in ((f, r["f"]), (psi, r["psi"])):
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isneginf(got), np.isneginf(ref))
+        assert np.abs(got[fin] - ref[fin]).max() <= solve_rtol(iters) * np.abs(ref[fin]).max()
