@@ -186,7 +186,8 @@ fot_status fot_solve_rect_fp64(const double* g, int rows_in, int cols_in, const 
  * spread of the potentials (u, V outside the FP32 range, or FFT rounding, a few ulp of a line's
  * largest value, swamping its small entries): a non-positive or non-finite convolution where
  * the marginal has mass latches FOT_ENONFINITE.  rows, cols in [2, 2048] (FFT length up to 4096;
- * else FOT_EUNSUPPORTED); iters >= 1.  Allocates a 32 KB spectrum buffer on its first call. */
+ * else FOT_EUNSUPPORTED); iters >= 1.  Allocates a 32 KB spectrum buffer and 128 KB of transform
+ * tables on its first call. */
 fot_status fot_cfot_solve(fot_ctx* ctx, const float* g, const float* G, double dx,
                           const double* eps, int n_eps, int eps_units, int iters);
 
@@ -234,7 +235,8 @@ fot_status fot_marginal_error(fot_ctx* ctx, double* l1_out, double* dual_out);
  * rows and cols must be powers of two in [2, 4096] (else FOT_EUNSUPPORTED); phi and loss_out
  * not NULL (else FOT_EINVAL); a problem loaded by fot_solve / fot_set_problem (else
  * FOT_ESTATE).  intensity_out (device, rows x cols, may be NULL) receives I.  Uses the
- * context's scratch buffers, not its potentials; FP32 transforms, FP64 sums.  Synchronising. */
+ * context's scratch buffers, not its potentials (and 128 KB of transform tables allocated by the
+ * first call); FP32 transforms, sums in FP64 and in pairs of FP32 numbers.  Synchronising. */
 fot_status fot_intensity_loss(fot_ctx* ctx, const float* phi, double* loss_out, float* intensity_out);
 
 /* One half-step from caller potentials, for verification and custom loops:

@@ -22,6 +22,7 @@ void set_problem_simt(fot_ctx* c, const float* g, const float* G, float* psi0, f
 void fill(fot_ctx* c, float* p, size_t N, float v);
 void source_stats(fot_ctx* c, const float* f, const float* S, double eps, double* out);
 bool intensity_supported(int rows, int cols);
+bool fft_tables(fot_ctx* c);
 bool cfot_supported(int rows, int cols);
 void cfot_run(fot_ctx* c, const double* eps_px, int iters);
 size_t cfot_spectrum_floats();
@@ -220,6 +221,7 @@ void fot_destroy(fot_ctx* c) {
     if (b) cudaFree(b);
   if (c->red) cudaFree(c->red);
   if (c->lam_hat) cudaFree(c->lam_hat);
+  if (c->roots) cudaFree(c->roots);
   if (c->err) cudaFree(c->err);
   if (c->terms) cudaFree(c->terms);
   if (c->ev_loop0) cudaEventDestroy(c->ev_loop0);
@@ -452,6 +454,7 @@ fot_status fot_cfot_solve(fot_ctx* c, const float* g, const float* G, double dx,
     c->lam_hat = nullptr;
     return FOT_ENOMEM;
   }
+  if (!fft_tables(c)) return FOT_ENOMEM;
   s = start_solve(c, g, G, dx, eps, eps_units);
   if (s != FOT_OK) return s;
   std::vector<double> e((size_t)iters);
@@ -642,16 +645,17 @@ fot_status fot_intensity_loss(fot_ctx* c, const float* phi, double* loss_out, fl
   if (!c->have_problem) return FOT_ESTATE;
   if (!intensity_supported(c->rows, c->cols)) return FOT_EUNSUPPORTED;
   FOT_CUDA(cudaSetDevice(c->device));
-  double* out = c->red + 4 * c->red_blocks + 8;      // [0] loss, [1] total power
+  if (!fft_tables(c)) return FOT_ENOMEM;
+  double* out = c->red + 4 * c->red_blocks + 8;
   intensity_loss_gpu(c, phi, out);
   if (intensity_out)
     FOT_CUDA(cudaMemcpyAsync(intensity_out, c->tmp, (size_t)c->rows * c->cols * sizeof(float),
                              cudaMemcpyDeviceToDevice, c->stream));
-  double h[2];
-  FOT_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+  double h = 0.0;
+  FOT_CUDA(cudaMemcpyAsync(&h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
   fot_status s = read_latched(c);
   if (s != FOT_OK) return s;
-  *loss_out = h[0];
+  *loss_out = h;
   return FOT_OK;
 }
 

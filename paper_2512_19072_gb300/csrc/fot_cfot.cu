@@ -6,10 +6,10 @@
 //
 // On its n outputs, the linear convolution of a line of length n with lambda equals the
 // circular convolution of length P >= 2n - 1 (a power of two) of the zero-padded line with
-// lambda wrapped around (lambda_j at index j mod P).  One CTA per line: a decimation-in-frequency
-// FFT leaves the padded line in bit-reversed order, where it is multiplied by lambda's spectrum
-// (real, lambda being even, and stored in that same order), and a decimation-in-time inverse FFT
-// returns natural order.  Pass 0 convolves the rows and writes them transposed; pass 1
+// lambda wrapped around (lambda_j at index j mod P).  The forward transform (fot_fft.cuh) leaves the
+// padded line in bit-reversed order, where it is multiplied by lambda's spectrum (real, lambda
+// being even, and stored in that same order), and the inverse one returns natural order; one CTA
+// holds one to eight lines.  Pass 0 convolves the rows and writes them transposed; pass 1
 // convolves the columns and applies the update (u = e^{log a} / y, and log y for S_last).
 //
 // FP32 throughout, like the exponential-domain iteration the paper's cFOT is: an FFT
@@ -19,88 +19,74 @@
 // marginal has mass latches FOT_ENONFINITE: the cFOT instability Sec. 5 reports at small eps.
 #include <math.h>
 
-#include "fot_common.cuh"
+#include "fot_fft.cuh"
 
 namespace fot {
 namespace {
 
-constexpr int kConvThreads = 256;
-constexpr int kConvMaxP = 4096;
+constexpr int kConvMaxP = kFftMax;
 
 __device__ __forceinline__ int bitrev(int i, int log2p) { return (int)(__brev((unsigned)i) >> (32 - log2p)); }
 
-// hat[bitrev(q)] = sum_{|j| <= n-1} lambda_j e^{-2 pi i j q / P} = 1 + 2 sum_{j >= 1} lambda_j cos(2 pi j q / P)
-__global__ void lambda_spectrum_kernel(float* __restrict__ hat, int n, int P, int log2p, double eps) {
+// hat[bitrev(q)] = sum_{|j| <= n-1} lambda_j e^{-2 pi i j q / P} = 1 + 2 sum_{j >= 1} lambda_j cos(2 pi j q / P),
+// in FP64: lambda_j once per CTA, the cosines from the table (an exponential and a cosine per term
+// took 100 us at n = 512)
+__global__ void __launch_bounds__(256) lambda_spectrum_kernel(float* __restrict__ hat, const double* __restrict__ cosines,
+                                                              int n, int P, int log2p, double eps) {
+  __shared__ double s_lam[256];
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= P) return;
+  const int step = kFftMax >> log2p;
   double acc = 1.0;
-  for (int j = 1; j < n; ++j) {
-    const double lam = exp(-(double)j * (double)j / (2.0 * eps));
-    if (lam == 0.0) break;                                    // decreasing in j
-    acc += 2.0 * lam * cospi(2.0 * (double)(((long long)j * q) % P) / (double)P);
+  for (int j0 = 0; j0 < n; j0 += 256) {
+    const int jt = j0 + threadIdx.x;
+    __syncthreads();
+    s_lam[threadIdx.x] = jt < n ? 2.0 * exp(-(double)jt * (double)jt / (2.0 * eps)) : 0.0;
+    __syncthreads();
+    if (s_lam[0] == 0.0) break;                               // decreasing in j
+    const int j1 = min(256, n - j0);
+    for (int j = j0 == 0 ? 1 : 0; j < j1; ++j)
+      acc += s_lam[j] * cosines[(((j0 + j) * q) & (P - 1)) * step];
   }
-  hat[bitrev(q, log2p)] = (float)acc;
+  if (q < P) hat[bitrev(q, log2p)] = (float)acc;
 }
 
 // PASS 0: y = (line of x) * lambda, written transposed: out[k][line].
 // PASS 1: y likewise, then out[k][line] = e^{lmarg} / y and logsum[k][line] = log y.
 template <int PASS>
-__global__ void __launch_bounds__(kConvThreads) conv_line_kernel(const float* __restrict__ x,
-                                                                 const float* __restrict__ hat,
-                                                                 float* __restrict__ out,
-                                                                 const float* __restrict__ lmarg,
-                                                                 float* __restrict__ logsum, int* err,
-                                                                 int n_lines, int n, int P, int log2p) {
-  __shared__ float s_re[kConvMaxP], s_im[kConvMaxP];
-  const int line = blockIdx.x;
-  const float* xl = x + (size_t)line * n;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    s_re[i] = i < n ? xl[i] : 0.f;
-    s_im[i] = 0.f;
+__global__ void __launch_bounds__(512) conv_line_kernel(const float* __restrict__ x, const float* __restrict__ hat,
+                                                        float* __restrict__ out, const float* __restrict__ lmarg,
+                                                        float* __restrict__ logsum, int* err,
+                                                        const float2* __restrict__ roots, int n_lines, int n,
+                                                        int log2p, int lpc) {
+  extern __shared__ float s_fft[];
+  const int P = 1 << log2p, tpl = P >> 3;
+  const int li = threadIdx.x % lpc, t = threadIdx.x / lpc;    // (lines in turn: see fot_fft.cu)
+  const int line = blockIdx.x * lpc + li;
+  const bool in = line < n_lines;
+  const float* xl = x + (size_t)min(line, n_lines - 1) * n;
+  float re[8], im[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int i = t + j * tpl;                                // n <= P / 2: the upper half is padding
+    re[j] = j < 4 && in && i < n ? xl[i] : 0.f;
+    im[j] = 0.f;
   }
-  // forward, decimation in frequency: pairs (i0, i0 + h) of each 2h block, twiddle e^{-i pi pos/h}
-  for (int h = P >> 1; h >= 1; h >>= 1) {
-    __syncthreads();
-    for (int b = threadIdx.x; b < (P >> 1); b += blockDim.x) {
-      const int pos = b & (h - 1);
-      const int i0 = ((b - pos) << 1) + pos, i1 = i0 + h;
-      float ws, wc;
-      sincospif(-(float)pos / (float)h, &ws, &wc);
-      const float ar = s_re[i0], ai = s_im[i0], br = s_re[i1], bi = s_im[i1];
-      s_re[i0] = ar + br;
-      s_im[i0] = ai + bi;
-      const float dr = ar - br, di = ai - bi;
-      s_re[i1] = dr * wc - di * ws;
-      s_im[i1] = dr * ws + di * wc;
-    }
+  float* const sm = s_fft + li * fft_line_stride(P, lpc);
+  fft_line<false>(re, im, log2p, t, roots, sm);
+  const float scale = 1.f / (float)P;                         // (a power of two: exact)
+  const float4 h0 = __ldg(reinterpret_cast<const float4*>(hat + 8 * t)), h1 = __ldg(reinterpret_cast<const float4*>(hat + 8 * t) + 1);
+  const float h[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    re[j] *= h[j];
+    im[j] *= h[j];
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {          // both in bit-reversed order
-    const float hq = hat[i];
-    s_re[i] *= hq;
-    s_im[i] *= hq;
-  }
-  // inverse, decimation in time from bit-reversed order: twiddle e^{+i pi pos/h}
-  for (int h = 1; h < P; h <<= 1) {
-    __syncthreads();
-    for (int b = threadIdx.x; b < (P >> 1); b += blockDim.x) {
-      const int pos = b & (h - 1);
-      const int i0 = ((b - pos) << 1) + pos, i1 = i0 + h;
-      float ws, wc;
-      sincospif((float)pos / (float)h, &ws, &wc);
-      const float tr = wc * s_re[i1] - ws * s_im[i1];
-      const float ti = wc * s_im[i1] + ws * s_re[i1];
-      const float ar = s_re[i0], ai = s_im[i0];
-      s_re[i1] = ar - tr;
-      s_im[i1] = ai - ti;
-      s_re[i0] = ar + tr;
-      s_im[i0] = ai + ti;
-    }
-  }
-  __syncthreads();
-  const float scale = 1.f / (float)P;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const float y = s_re[k] * scale;
+  fft_line<true>(re, im, log2p, t, roots, sm);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = t + j * tpl;
+    if (!in || k >= n) continue;
+    const float y = re[j] * scale;
     const size_t o = (size_t)k * n_lines + line;
     if (PASS == 0) {
       out[o] = y;
@@ -130,8 +116,8 @@ __global__ void to_potential_kernel(float* __restrict__ p, size_t N, float eps) 
   }
 }
 
-int pad_log2(int n) {                 // log2 of the smallest power of two >= 2n - 1
-  int l = 0;
+int pad_log2(int n) {                 // log2 of the smallest power of two >= max(2n - 1, 8)
+  int l = 3;
   while ((1 << l) < 2 * n - 1) ++l;
   return l;
 }
@@ -155,11 +141,14 @@ void cfot_run(fot_ctx* c, const double* eps_px, int iters) {
   fill_value_kernel<<<fill_blocks, 256, 0, c->stream>>>(c->psi, N, (float)(1.0 / ((double)nr * nc)));
   int64_t k = 1;
   double e_prev = -1.0;
+  const int lpc_c = fft_lines_per_cta(Pc, nr), lpc_r = fft_lines_per_cta(Pr, nc);   // lines of nc values, of nr values
+  const size_t sm_c = (size_t)lpc_c * fft_line_stride(Pc, lpc_c) * sizeof(float);
+  const size_t sm_r = (size_t)lpc_r * fft_line_stride(Pr, lpc_r) * sizeof(float);
   for (int t = 0; t < iters; ++t) {
     const double e = eps_px[t];
     if (e != e_prev) {
-      lambda_spectrum_kernel<<<(Pr + 255) / 256, 256, 0, c->stream>>>(hat_r, nr, Pr, lr, e);
-      lambda_spectrum_kernel<<<(Pc + 255) / 256, 256, 0, c->stream>>>(hat_c, nc, Pc, lc, e);
+      lambda_spectrum_kernel<<<(Pr + 255) / 256, 256, 0, c->stream>>>(hat_r, c->cosines, nr, Pr, lr, e);
+      lambda_spectrum_kernel<<<(Pc + 255) / 256, 256, 0, c->stream>>>(hat_c, c->cosines, nc, Pc, lc, e);
       k += 2;
       e_prev = e;
     }
@@ -168,10 +157,10 @@ void cfot_run(fot_ctx* c, const double* eps_px, int iters) {
       float* outp = half == 0 ? c->f : c->psi;           // u, then V
       const float* lm = half == 0 ? c->la : c->lb;
       float* ls = (half == 0 && t == iters - 1) ? c->S_last : nullptr;
-      conv_line_kernel<0><<<nr, kConvThreads, 0, c->stream>>>(in, hat_c, c->R, nullptr, nullptr, c->err, nr, nc,
-                                                              Pc, lc);
-      conv_line_kernel<1><<<nc, kConvThreads, 0, c->stream>>>(c->R, hat_r, outp, lm, ls, c->err, nc, nr, Pr,
-                                                              lr);
+      conv_line_kernel<0><<<(nr + lpc_c - 1) / lpc_c, lpc_c * (Pc / 8), sm_c, c->stream>>>(
+          in, hat_c, c->R, nullptr, nullptr, c->err, c->roots, nr, nc, lc, lpc_c);
+      conv_line_kernel<1><<<(nc + lpc_r - 1) / lpc_r, lpc_r * (Pr / 8), sm_r, c->stream>>>(
+          c->R, hat_r, outp, lm, ls, c->err, c->roots, nc, nr, lr, lpc_r);
       k += 2;
     }
   }

@@ -79,6 +79,10 @@ struct fot_ctx {
   float* col_phi = nullptr;  // rows: phase along the centre column
   float* plan = nullptr;     // per-(row, 16-output tile) window plan of a banded pass, 3 words each
   double* red = nullptr;     // reduction scratch (partials + results)
+  // tables of the transforms (one allocation, made by the first one) and their partial sums
+  float2* roots = nullptr;
+  double* cosines = nullptr;
+  double* fft_parts = nullptr;
   float* lam_hat = nullptr;  // cFOT: the spectra of lambda (allocated by the first cFOT solve)
   int* err = nullptr;        // latched device status
   unsigned long long* terms = nullptr;  // device counters of evaluated (row, output, m) terms
