@@ -167,10 +167,10 @@ fot_status fot_create(fot_ctx** out, int rows, int cols, int precision, int devi
   bool ok = true;
   for (float** b : bufs) ok = ok && cudaMalloc((void**)b, N * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->col_phi, (size_t)rows * sizeof(float)) == cudaSuccess;
-  // the per-(16-output tile, row) plan of the larger banded pass (3 words each; rows padded to
+  // the per-(tile, row) plan of the larger banded pass (3 words each; rows padded to
   // a multiple of 8, the plan's tile-major stride)
   const size_t pr = (size_t)(rows + 7) / 8 * 8, pc = (size_t)(cols + 7) / 8 * 8;
-  const size_t plan_words = 3 * std::max(pr * ((cols + 15) / 16), pc * ((rows + 15) / 16));
+  const size_t plan_words = 3 * std::max(pr * plan_tiles(cols), pc * plan_tiles(rows));
   ok = ok && cudaMalloc((void**)&c->plan, plan_words * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->red, (size_t)(4 * c->red_blocks + 16) * sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->err, sizeof(int)) == cudaSuccess;
@@ -186,8 +186,8 @@ fot_status fot_create(fot_ctx** out, int rows, int cols, int precision, int devi
   }
   if (precision == FOT_MIXED || precision == FOT_BF16)
     ok = ok && cudaMalloc((void**)&c->tilt, tilt_bytes()) == cudaSuccess;
-  // items of the window kernel: groups of 8 rows x 4 tiles of at least 16
-  const size_t n_items = std::max(pr / 8 * ((cols + 63) / 64), pc / 8 * ((rows + 63) / 64));
+  // items of the window kernel: groups of 8 rows x 4 tiles
+  const size_t n_items = std::max(pr / 8 * ((plan_tiles(cols) + 3) / 4), pc / 8 * ((plan_tiles(rows) + 3) / 4));
   ok = ok && cudaMalloc((void**)&c->items, n_items * sizeof(int4)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&c->order, 2 * sizeof(int)) == cudaSuccess;
   if (ok) ok = cudaMemsetAsync(c->order, 0, 2 * sizeof(int), c->stream) == cudaSuccess;

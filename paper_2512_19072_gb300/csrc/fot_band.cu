@@ -16,7 +16,6 @@
 //    at its nearest distance to the tile) lies below LB - kCut holds only terms below 2^-kCut
 //    of every output of the tile; the window is the hull of the remaining blocks (found per
 //    32-wide chunk first, then narrowed from both ends).
-// 3. Whether the row's operands stay in range for the tilted product (row_in_range).
 // Arg-maxima carry the index in the low mantissa bits of the value they compare (5 bits for a
 // position, 7 for a chunk): one maximum instead of a compare and two selects; a chunk's maximum
 // is rounded by 2^-18 of itself that way, far inside the margin of kCut.
@@ -126,7 +125,6 @@ __global__ void __launch_bounds__(kPlanThreads) band_plan_kernel(const __grid_co
   const size_t np = (size_t)a.plan_stride * T;
   int* const plan_i = reinterpret_cast<int*>(a.plan);
   const int q = ti & (kPlanQ - 1);
-  const float kmax = 0.5f * (float)tw;
   const f32x2 nc2 = pack2(-c, -c);
   // (lanes past the tiles or rows compute on a valid place and write nothing: the shuffles below
   // want whole warps)
@@ -240,11 +238,10 @@ __global__ void __launch_bounds__(kPlanThreads) band_plan_kernel(const __grid_co
     if (has && q == 0) {
       const int lo = win ? edge * 8 : 0, hi = win ? min(other * 8, len) : 0;
       mh = max(lo, min(mh, hi - 1));
-      const bool in = !win || row_in_range(kmax, lo, hi, mh, c);
       const size_t pi = (size_t)t * a.plan_stride + row;
       a.plan[pi] = any ? alpha : -INFINITY;
       plan_i[np + pi] = lo | ((hi - lo) << 16);
-      plan_i[2 * np + pi] = mh | (in ? 0 : 1 << 16);
+      plan_i[2 * np + pi] = mh;
       if (hi > lo) {
         atomicMin(&s_lo[t / kWinWarps], lo);
         atomicMax(&s_hi[t / kWinWarps], hi);
@@ -297,15 +294,19 @@ void finish(BandTable<MAXP>& t, int* max_chunks) {
 }  // namespace
 
 // Tile width for a problem with kernel constant c.  A row's operands stay in range while
-// tile_w (D + mh - lo) c <= kRangeMax, D the farthest window position from mh.  For a smooth
+// tile_w (D + mh - lo) c <= kRangeMax = 100, D the farthest window position from mh.  For a smooth
 // potential the window W is about the tile plus the distance sqrt(kCut / c) on both sides at which
-// the Gaussian has fallen by 2^-kCut, with mh in its middle: tile_w W c.  The limit for 32 leaves
-// room for windows half as wide again (rows outside the bound cost more there).  The wider tile
-// shares each exponential, and each unit's set-up, between more outputs.
+// the Gaussian has fallen by 2^-kCut, with mh in its middle: tile_w W c.  Real windows are longer
+// where the transport map jumps, so a width is taken while that estimate leaves room (the wider
+// tile shares each exponential, and each unit's set-up, between more outputs; units out of range
+// are summed in segments).  8 ends where exact sums become the faster ones (at 256^2, per pass:
+// eps 7 12.7 against 23.5 us, eps 5 13.0 against 10.3).
 int tile_width_for(float c) {
   const float reach = 2.f * sqrtf(kCut / c);
-  if (32.f * (32.f + reach) * c <= 70.f) return 32;
-  if (16.f * (16.f + reach) * c <= 100.f) return 16;
+  auto need = [&](float w) { return w * (w + reach) * c; };
+  if (need(32.f) <= 42.f) return 32;
+  if (need(16.f) <= 64.f) return 16;
+  if (need(8.f) <= 45.f) return 8;
   return 0;
 }
 
@@ -317,7 +318,7 @@ void band_set_eps(BandArgs& a, double eps) {
   a.group = tw == 0 ? 2 : 8;
   a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
   if (tw != 0)
-    for (int i = 0; i < 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
+    for (int i = 0; i <= 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
 }
 
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale) {
@@ -359,7 +360,11 @@ template <int MODE, int MAXP>
 void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
   plan_pass(s, t);
   ktimer_begin(s, form == kFormFp32 ? kKBand : kKTensor);
-  if (form == kFormFp32)
+  bool exact = true;
+  for (int q = 0; q < t.n; ++q) exact = exact && t.p[q].group == 2;
+  if (exact)
+    exact_launch<MODE, MAXP>(s, t);
+  else if (form == kFormFp32)
     window_launch<MODE, kFormFp32, MAXP>(s, t);
   else if (form == kFormSplit)
     window_launch<MODE, kFormSplit, MAXP>(s, t);
@@ -375,7 +380,7 @@ template void band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
 
 // the plan kernel stages eight rows: more than the default 48 KB from rows of 1152 on
 cudaError_t plan_configure() {
-  const int lim = (int)(kPlanRows * plan_row_floats(4096 / kCW) * sizeof(float)) + 2 * 64 * (int)sizeof(int);
+  const int lim = (int)(kPlanRows * plan_row_floats(4096 / kCW) * sizeof(float)) + 2 * 256 * (int)sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(band_plan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(band_plan_kernel<kMaxBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -427,7 +432,7 @@ void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
     if (!c->tilt_eps.empty() && c->tilt_eps.back() == eps[i]) continue;
     const float cc = (float)(1.4426950408889634 / (2.0 * eps[i]));
     const int tw = tile_width_for(cc);
-    if (tw == 0) continue;                    // exact windows only: no table
+    if (tw < 16) continue;                    // narrow tiles, exact windows: no table
     const int k = (int)c->tilt_eps.size();
     t.c[k] = cc;
     t.tw[k >> 2] |= tw << (8 * (k & 3));
@@ -441,7 +446,7 @@ void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
 }
 
 const uint4* tilt_for(fot_ctx* c, double eps, int tile_w, int64_t* launches) {
-  if (!c->tilt || tile_w == 0) return nullptr;
+  if (!c->tilt || tile_w < 16) return nullptr;
   for (size_t i = 0; i < c->tilt_eps.size(); ++i)
     if (c->tilt_eps[i] == eps) return c->tilt + i * kTiltWords;
   tilt_prepare(c, &eps, 1, launches);

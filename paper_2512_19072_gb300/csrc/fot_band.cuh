@@ -14,8 +14,7 @@ enum WindowForm : int { kFormFp32 = 0, kFormSplit = 1, kFormSingle = 2 };
 // One problem's pass over rows of x: y[o][r] = log2 sum_m 2^(x[r][m] x_scale - (o + shift - m)^2 c).
 // plan holds, per (tile of tile_w outputs, row) at t * plan_stride + r, three arrays of
 // n_tiles * plan_stride words each: the offset alpha (float), the window start | length << 16
-// (positions) and mh | flag << 16 (the position the offset was taken at; the flag marks a row whose
-// operands leave the range of the tilted product, fot_window.cuh).
+// (positions) and mh, the position the offset was taken at.
 struct BandArgs {
   const float* x;      // [n_rows][len] input
   float* plan;
@@ -37,7 +36,7 @@ struct BandArgs {
   float coord0, coord_step;
   float x_scale, c, eps, shift;
   int n_rows, len, n_out;
-  int tile_w;          // outputs per plan tile and window unit: 16 or 32
+  int tile_w;          // outputs per plan tile and window unit: 8, 16 or 32
   int group;           // rows per window unit: 8, or 2 where every unit takes exact window sums
   int n_chunks, n_tiles, plan_stride;
   int plan_base, item_base;    // first plan CTA and first window item of this problem
@@ -45,7 +44,7 @@ struct BandArgs {
   int wide_span;               // items whose windows span more go first
   int vec;                     // bit 0: rows of x are 16-byte aligned; bit 1: pairs of outputs are
                                // 8-byte aligned
-  float step[32];              // 2^(32 kap c), kap = i - 16: the accumulators' scale per window
+  float step[33];              // 2^(32 kap c), kap = i - 16: the accumulators' scale per window
                                // step, rounded once from 64 bits (its error grows with the steps)
 };
 
@@ -83,10 +82,13 @@ __device__ __forceinline__ int find_prob(const BandTable<MAXP>& t, int gi) {
   return lo;
 }
 
-// Tile width of a pass with kernel constant c: outputs per window unit, 32 or 16; 0 where no
-// unit can take the tilted GEMM (the pass then runs exact window sums in units of 2 rows x 16
+// Tile width of a pass with kernel constant c: outputs per window unit, 32, 16 or 8; 0 where
+// eps is too small for the tilted product (the pass then runs exact window sums in units of 2 rows x 16
 // outputs).
 int tile_width_for(float c);
+
+// tiles of n outputs that a plan must have room for: 8-wide ones
+inline size_t plan_tiles(int n) { return ((size_t)n + 7) / 8; }
 
 // the fields of a pass that follow from eps: kernel constant, tile width, step scales
 void band_set_eps(BandArgs& a, double eps);

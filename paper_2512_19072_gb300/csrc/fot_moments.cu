@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) moment_pass_kernel(const __gri
     return;
   }
   const int W = __reduce_max_sync(0xffffffffu, rv.wl);
-  if (!__any_sync(0xffffffffu, u.out_of_range)) {
+  if (unit_walk(8.f, rv, W, a.c) == 0) {
     if (lane == 0 && W > 0) atomicAdd(terms, (unsigned long long)W * 16 * 8);
     if (moment_unit<MODE>(a, u.r0, u.k0, (float)(u.k0 + 8) + a.shift, rv, u.row, W, tilt, u.skip)) return;
   }
@@ -224,7 +224,9 @@ __global__ void __launch_bounds__(kWinThreads, 4) moment_pass_kernel(const __gri
 
 template <int MODE>
 void moment_pass(fot_ctx* c, BandTable<1>& t) {
-  t.p[0].tile_w = 16;                                     // (group: as the half-steps')
+  const float reach = 2.f * sqrtf(kCut / t.p[0].c);
+  t.p[0].tile_w = 16;
+  t.p[0].group = 16.f * (16.f + reach) * t.p[0].c <= 64.f ? 8 : 2;
   t.p[0].wide_span = kWinWarps * 16 + (int)(2.6f * sqrtf(kCut / t.p[0].c));
   plan_pass(c->stream, t);
   launch_dependent(moment_pass_kernel<MODE>, dim3(t.items), kWinThreads, window_smem(t.pitch_max), c->stream, t);

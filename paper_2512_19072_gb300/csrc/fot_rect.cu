@@ -185,8 +185,8 @@ fot_status solve_rect(const T* g, int rows_in, int cols_in, const T* G, int rows
     const int pass[4][2] = {{rows_out, cols_in}, {cols_in, rows_in}, {rows_in, cols_out}, {cols_out, rows_out}};   // rows, outputs
     for (const int(&p)[2] : pass) {
       const size_t r8 = (size_t)(p[0] + 7) / 8 * 8;
-      plan_words = std::max(plan_words, 3 * r8 * ((p[1] + 15) / 16));
-      n_items = std::max(n_items, r8 / 8 * ((p[1] + 63) / 64));
+      plan_words = std::max(plan_words, 3 * r8 * plan_tiles(p[1]));
+      n_items = std::max(n_items, r8 / 8 * ((plan_tiles(p[1]) + 3) / 4));
     }
   }
   size_t need = 0;

@@ -29,33 +29,46 @@
 //
 // Horner over 16-position steps.  T[kap][p + 16] = T[kap][p] 2^(32 kap c): moving the reference
 // by one step scales row kap by a constant.  So the operand fragments of T for one step stay in
-// registers for the whole window, which is walked from its end to its start; the sums D become
-// D G + (the step's products), G = 2^(32 kap c), and end up referred to lo_r.  The products start
-// from zero and are added by the CUDA cores: the tensor core truncates what it accumulates, and
-// a chain of steps through it added up to 1e-5 of a sum.  Two steps per turn of the loop, their
-// products added a turn later, so that the exponentials of one turn run while the tensor core
-// works on the last: a long window is one warp's chain (45 steps at 1024^2 where the mean is 13).
+// registers for the whole window, which is walked down to its start or up to its end; the sums D
+// become D G + (the step's products), G = 2^(+-32 kap c), and end up referred to the first position
+// of the last step walked.  The products start from zero and are added by the CUDA cores: the
+// tensor core truncates what it accumulates, and a chain of steps through it added up to 1e-5 of a
+// sum.  Two steps per turn of the loop, their products added a turn later, so that the exponentials
+// of one turn run while the tensor core works on the last: a long window is one warp's chain (45
+// steps at 1024^2 where the mean is 13).
 //
 // Operands.  kFormSplit: BF16 hi + lo parts, hi*hi + hi*lo + lo*hi (2^-16 relative per product);
 // kFormSingle: hi*hi; kFormFp32: TF32 hi + lo parts (2^-21), two m16n8k8 per step and product.
 //
 // Range.  With kmax = TN/2 and D the farthest window position from mh: a term that matters to
 // output kap has X >= 2^-(2 kmax D c) (alpha is e(mh, kc); the largest term at kap is at least
-// mh's), and referring the sum to lo_r instead of mh moves it by at most 2 kmax (mh - lo_r) c.  A
+// mh's), and referring the sum to position r instead of mh moves it by at most 2 kmax |mh - r| c.  A
 // row is in range while the first is <= kTiltMax and both together are <= kRangeMax: what flushes
 // to zero below 2^-126 is then less than W 2^-30 of a sum, and sums stay below 2^(100 + 9) times
-// 2^(how far the offset lies below the maximum).  An offset that lies too far below shows as an
-// output that is not finite; such a unit is summed again exactly.
+// 2^(how far the offset lies below the maximum).  The walk ends at the start of the window where
+// every row is in range that way, else at its end (mh sits at one end of most windows that span a
+// gap).  An offset that lies too far below the maximum shows as an output that is not finite; such a
+// unit is summed again in segments.
 //
-// Units outside that bound: a 32-wide tile is cut in two 16-wide ones that take their own
-// offsets; what fails again (or a problem whose eps is too small for any unit) is summed exactly:
-// one exponential per term and output, lanes on 2 rows x 16 outputs, offset e(mh, o).
+// Narrow tiles.  The range shrinks with the tile: where eps is too small for 16 outputs, tiles of 8
+// take the same product with the unused rows of T zero, always with FP32 operands.  Below that
+// (eps < 5) every output is summed exactly, one exponential per term, relative to e(mh, o), by a
+// kernel of its own (exact_pass_kernel): its windows are a few blocks long, and tiles of 4 with the
+// product were slower (256^2, eps 1: 16.6 against 11.5 us per pass; 64^2: 10.7 against 6.2).
+//
+// Segments.  A unit outside the bound (a window that spans the gap between two parts of a target,
+// mostly) is summed with FP32 operands in segments of its window short enough to be in range by
+// themselves, each with its rows' maxima as offsets; the segments' sums are added as logarithms, and a segment in
+// which no row has a term within 2^-kCut of its output's largest is passed over.  (Exact sums for
+// these units, one in twenty, made a pass at 256^2 and eps 15 three times as long: 18.6 us, 13.4 with
+// segments.)  What fails even then is summed exactly.
 //
 // What bounds it: issue slots and latency.  A split-BF16 step at TN = 32 is about 40 instructions
 // and 6 MMAs (48 tensor cycles per SM quarter), a unit's set-up and outputs about 450.  A loop of
-// 200 iterations at 1024^2 (800 passes, plan and launch gaps included): split BF16 31.9 -> 16.6 ms,
-// FP32 45.7 -> 18.4 ms (it was FFMA with the operands through shared memory); 100 iterations at
-// 2048^2, split BF16: 39.8 -> 20.9 ms; 64^2 at eps 1 (exact windows), 200 iterations: 14.5 -> 4.5 ms.
+// 200 iterations at 1024^2 (800 passes, plan and launch gaps included) went from 31.9 to 14.5 ms with
+// split BF16 and from 45.7 to 16.5 ms with FP32 operands (FFMA with the operands through shared memory
+// before); 100 iterations at 2048^2, split BF16, from 39.8 to 21.2 ms; 256^2 annealed from eps 64 to 1
+// over 300 iterations from 41.7 to 11.7 ms; 64^2 at eps 1, 200 iterations, from 14.5 to 4.6 ms.
 #pragma once
 
 #include "fot_band.cuh"
@@ -270,7 +283,8 @@ struct Tilt {
   static constexpr int NH = FORM == kFormFp32 ? 2 : 1;
   uint32_t hi[2][4 * NH], lo[2][4 * NH];
   f32x2 G[2][2];
-  // tw = 16 (first row tile only) or 32; table: a.tilt holds the fragments (BF16 forms)
+  // tw: outputs of the tile (16 and 8: first row tile only, 8: its second half zero); table:
+  // a.tilt holds the fragments (BF16 forms, tiles of 16 and 32)
   __device__ __forceinline__ void load(const BandArgs& a, int tw, bool table) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -279,7 +293,12 @@ struct Tilt {
       const int kap0 = 16 * t - tw / 2;
       if (FORM == kFormFp32) {
 #pragma unroll
-        for (int h = 0; h < NH; ++h) tilt_fragments_tf32(a.c, kap0, h, lane, hi[t] + 4 * h, lo[t] + 4 * h);
+        for (int h = 0; h < NH; ++h) {
+          tilt_fragments_tf32(a.c, kap0, h, lane, hi[t] + 4 * h, lo[t] + 4 * h);
+          if (tw < 16) {
+            hi[t][4 * h + 1] = hi[t][4 * h + 3] = lo[t][4 * h + 1] = lo[t][4 * h + 3] = 0u;
+          }
+        }
       } else if (table) {
         const uint4 h4 = __ldg(a.tilt + t * 64 + lane), l4 = __ldg(a.tilt + t * 64 + 32 + lane);
         hi[t][0] = h4.x; hi[t][1] = h4.y; hi[t][2] = h4.z; hi[t][3] = h4.w;
@@ -289,28 +308,32 @@ struct Tilt {
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float v = a.step[kap0 + (lane >> 2) + 8 * h + 16];
+        const float v = a.step[min(kap0 + (lane >> 2) + 8 * h, 15) + 16];
         G[t][h] = pack2(v, v);
       }
     }
   }
 };
 
-// The tilted matrix product of one unit (see the top).  Lane (g = lane / 4, q = lane % 4) owns row
-// r0 + g (rv) for X, and outputs kap g and g + 8 of each row tile of columns r0 + 2q, + 1.
-// Returns false, with nothing written, when a sum left the range of FP32 (warp-uniform).
-template <int MODE, int FORM, int TN, bool STAGED>
-__device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, float kc, const RowView& rv, int W,
-                                          const Tilt<FORM>& tilt, bool skip) {
-  constexpr int MT = TN / 16;
+// The window sums D of one unit (see the top), referred to each row's lo (up: to the first position
+// of the last step, lo + walk_end(W)).  Lane (g = lane / 4, q = lane % 4) owns row g of the unit (rv)
+// for X, and outputs kap g and g + 8 of each row tile of columns 2q, 2q + 1.
+__device__ __forceinline__ bool long_window(int W, float c) {  // so much longer than a smooth potential's
+  return (float)W * (float)W * c > 900.f;                 // (about 210) that it is likely to span a gap
+}
+__device__ __forceinline__ int walk_end(int W) { return ((W + 31) >> 5) * 32 - 16; }
+// PLAIN: the common case, rows staged, walking down, no look for empty turns (fewer registers).
+template <int FORM, int TN, bool PLAIN>
+__device__ __forceinline__ void window_product(const BandArgs& a, float kc, const RowView& rv, int W, bool up_,
+                                               const Tilt<FORM>& tilt, f32x2 (&D)[TN < 16 ? 1 : TN / 16][2]) {
+  constexpr int MT = TN < 16 ? 1 : TN / 16;
   constexpr int NH = Tilt<FORM>::NH;
-  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int q = threadIdx.x & 3;
   const float c = a.c;
   const float sc = a.x_scale;
   const f32x2 sc2 = pack2(sc, sc), nc2 = pack2(-c, -c);
   const float na = rv.wl == 0 ? 0.f : -rv.alpha;
   const f32x2 na2 = pack2(na, na);
-  f32x2 D[MT][2];                                         // (columns 2q, 2q + 1) of rows g and g + 8
   float P[2][MT][4];                                      // the last turn's products
 #pragma unroll
   for (int t = 0; t < MT; ++t) {
@@ -318,22 +341,36 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
 #pragma unroll
     for (int u = 0; u < 4; ++u) P[0][t][u] = P[1][t][u] = 0.f;
   }
+  const bool up = !PLAIN && up_;
   const int turns = (W + 31) >> 5;
-  int pos = rv.lo + 32 * turns - 16 + 4 * q;              // this lane's first position of the step
-  int left = rv.wl - 32 * turns + 16 - 4 * q;             // of it and after it in the window
+  const int first = up ? 0 : walk_end(W), by = up ? 16 : -16;
+  int pos = rv.lo + first + 4 * q;                        // this lane's first position of the step
+  int left = rv.wl - first - 4 * q;                       // of it and after it in the window
   uint32_t addr = rv.saddr + 4u * (uint32_t)pos;
   const float d0 = kc - (float)pos;
   f32x2 d01 = pack2(d0, d0 - 1.f);
-  const f32x2 d16 = pack2(16.f, 16.f);
+  const f32x2 d16 = pack2((float)-by, (float)-by);
+  f32x2 G[MT][2];
+#pragma unroll
+  for (int t = 0; t < MT; ++t)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      G[t][h] = tilt.G[t][h];
+      if (up) {
+        const float v = a.step[16 - (16 * t - TN / 2 + (int)((threadIdx.x & 31) >> 2) + (TN < 16 ? 0 : 8 * h))];
+        G[t][h] = pack2(v, v);
+      }
+    }
+  const bool gaps = !PLAIN && long_window(W, c);
   auto fetch = [&]() {
     float4 v;
-    if (STAGED)
+    if (PLAIN)
       v = lds4(left > 0 ? addr : rv.minf);
     else
       v = fetch4(rv.row, pos, left, rv.vec);
-    addr -= 64u;
-    pos -= 16;
-    left += 16;
+    addr += (uint32_t)(4 * by);
+    pos += by;
+    left -= by;
     return v;
   };
   auto absorb = [&]() {                                   // D <- (D G + P0) G + P1
@@ -341,8 +378,8 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int t = 0; t < MT; ++t) {
-        D[t][0] = fma2(D[t][0], tilt.G[t][0], pack2(P[i][t][0], P[i][t][1]));
-        D[t][1] = fma2(D[t][1], tilt.G[t][1], pack2(P[i][t][2], P[i][t][3]));
+        D[t][0] = fma2(D[t][0], G[t][0], pack2(P[i][t][0], P[i][t][1]));
+        D[t][1] = fma2(D[t][1], G[t][1], pack2(P[i][t][2], P[i][t][3]));
       }
   };
   float4 xn[2];
@@ -357,20 +394,43 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
       xn[0] = fetch();
       xn[1] = fetch();
     }
+    float e[2][4];
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      exponents4(xv[v], sc2, na2, nc2, d01, e[v]);
+      d01 = add2(d01, d16);
+    }
+    if (gaps) {
+      // a turn whose operands are all zero (ex2 flushes below 2^-126).  As unsigned words, the
+      // numbers below -126 are those above its own (a NaN of the arithmetic, 0x7fffffff, is not:
+      // it takes the products)
+      uint32_t least = 0xffffffffu;
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) least = min(least, __float_as_uint(e[v][u]));
+      if (__all_sync(0xffffffffu, least > 0xc2fc0000u)) {
+        absorb();
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int t = 0; t < MT; ++t)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) P[v][t][u] = 0.f;
+        continue;
+      }
+    }
     uint32_t xh[2][2 * NH], xl[2][2 * NH];
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
-      float e[4];
-      exponents4(xv[v], sc2, na2, nc2, d01, e);
-      d01 = add2(d01, d16);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) e[u] = ex2(e[u]);
+      for (int u = 0; u < 4; ++u) e[v][u] = ex2(e[v][u]);
       if (FORM == kFormFp32) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) split_tf32(e[u], xh[v][u % (2 * NH)], xl[v][u % (2 * NH)]);
+        for (int u = 0; u < 4; ++u) split_tf32(e[v][u], xh[v][u % (2 * NH)], xl[v][u % (2 * NH)]);
       } else {
-        split_bf16(e[0], e[1], xh[v][0], xl[v][0]);
-        split_bf16(e[2], e[3], xh[v][1], xl[v][1]);
+        split_bf16(e[v][0], e[v][1], xh[v][0], xl[v][0]);
+        split_bf16(e[v][2], e[v][3], xh[v][1], xl[v][1]);
       }
     }
     absorb();
@@ -390,50 +450,51 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
           }
   }
   absorb();
+}
 
-  // outputs of columns rA = r0 + 2q and rA + 1; an empty row (alpha = -inf) has sums 0: log -inf
+// Outputs of a unit: the log-sum of output group i (kap = 8 i - TN/2 + g) and column u is
+// al[u] + t[i][u].  False, with nothing written, when one is not finite where its row has mass
+// (warp-uniform).
+template <int MODE, int TN>
+__device__ __forceinline__ bool write_unit(const BandArgs& a, int r0, int k0, const float (&al)[TN < 16 ? 1 : TN / 8][2],
+                                           const float (&t)[TN < 16 ? 1 : TN / 8][2], bool skip) {
+  constexpr int NO = TN < 16 ? 1 : TN / 8;                // groups of up to 8 outputs
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int rA = r0 + 2 * q;
-  const float al[2] = {__shfl_sync(0xffffffffu, rv.alpha, 8 * q), __shfl_sync(0xffffffffu, rv.alpha, 8 * q + 4)};
-  const float mr[2] = {(float)__shfl_sync(0xffffffffu, rv.lo, 8 * q) - kc,
-                       (float)__shfl_sync(0xffffffffu, rv.lo, 8 * q + 4) - kc};   // reference - kc
   const size_t y0 = (size_t)(k0 + g) * a.n_rows + rA;
   const size_t ystep = (size_t)8 * a.n_rows;
   const bool full = (a.vec & 2) && k0 + TN <= a.n_out && r0 + 8 <= a.n_rows;   // warp-uniform
-  float lm[2 * MT][2];
+  auto inside = [&](int i) { return k0 + g + 8 * i < a.n_out; };
+  float lm[NO][2];
   if (MODE == 1) {
 #pragma unroll
-    for (int i = 0; i < 2 * MT; ++i) {
+    for (int i = 0; i < NO; ++i) {
       const float* p = a.lmarg + y0 + i * ystep;
       if (full) {
         const float2 v = __ldg(reinterpret_cast<const float2*>(p));
         lm[i][0] = v.x;
         lm[i][1] = v.y;
       } else {
-        const bool in = k0 + g + 8 * i < a.n_out;
+        const bool in = inside(i);
         lm[i][0] = in && rA < a.n_rows ? __ldg(p) : -INFINITY;
         lm[i][1] = in && rA + 1 < a.n_rows ? __ldg(p + 1) : -INFINITY;
       }
     }
   }
-  float s2[2 * MT][2], chk[2] = {0.f, 0.f};               // chk: NaN after a non-finite log-sum
+  float s2[NO][2], chk[2] = {0.f, 0.f};                   // chk: NaN after a non-finite log-sum
 #pragma unroll
-  for (int i = 0; i < 2 * MT; ++i) {
-    const float kap = (float)(8 * i - TN / 2 + g);
-    float v[2];
-    unpack2(D[i >> 1][i & 1], v[0], v[1]);
+  for (int i = 0; i < NO; ++i)
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const float l2 = FORM == kFormFp32 ? log2f(v[u]) : lg2(v[u]);
-      s2[i][u] = __fadd_rn(al[u], fmaf(fmaf(2.f * kap, mr[u], -kap * kap), c, l2));
+      s2[i][u] = __fadd_rn(al[i][u], t[i][u]);
       chk[u] = fmaf(s2[i][u], 0.f, chk[u]);
     }
-  }
-  if (__any_sync(0xffffffffu, (chk[0] != 0.f && al[0] != -INFINITY) || (chk[1] != 0.f && al[1] != -INFINITY)))
+  if (__any_sync(0xffffffffu, (chk[0] != 0.f && al[0][0] != -INFINITY) || (chk[1] != 0.f && al[0][1] != -INFINITY)))
     return false;
   if (skip) return true;
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < 2 * MT; ++i) {
+  for (int i = 0; i < NO; ++i) {
     float out[2], sv[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) out[u] = finish_output<MODE>(a, s2[i][u], MODE == 1 ? lm[i][u] : 0.f, sv[u], bad);
@@ -441,7 +502,7 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
     if (full) {
       *reinterpret_cast<float2*>(a.y + yi) = make_float2(out[0], out[1]);
       if (MODE == 1 && a.logsum) *reinterpret_cast<float2*>(a.logsum + yi) = make_float2(sv[0], sv[1]);
-    } else if (k0 + g + 8 * i < a.n_out) {
+    } else if (inside(i)) {
 #pragma unroll
       for (int u = 0; u < 2; ++u)
         if (rA + u < a.n_rows) {
@@ -454,14 +515,47 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
   return true;
 }
 
-// Exact window sums of 2 rows x 16 outputs: lane (half, i) owns output k0 + i of its half's row,
-// window [lo, lo + wl), xp[m] that row's position m.  Terms are taken relative to e(mh, o), which
-// is within the range of FP32 of the maximum unless the maximum moves far from mh within the
-// tile; a sum that overflows is done again from its exact maximum.
+// log-sums of the sums D (referred to lo + ref): offset and rest of every output
+template <int FORM, int TN>
+__device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowView& rv, int ref,
+                                         const f32x2 (&D)[TN < 16 ? 1 : TN / 16][2], float (&al)[TN < 16 ? 1 : TN / 8][2],
+                                         float (&t)[TN < 16 ? 1 : TN / 8][2]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const float alpha = __shfl_sync(0xffffffffu, rv.alpha, 8 * q + 4 * u);
+    const float mr = (float)(__shfl_sync(0xffffffffu, rv.lo, 8 * q + 4 * u) + ref) - kc;   // reference - kc
+#pragma unroll
+    for (int i = 0; i < (TN < 16 ? 1 : TN / 8); ++i) {
+      const float kap = (float)(8 * i - TN / 2 + g);
+      float v[2];
+      unpack2(D[i >> 1][i & 1], v[0], v[1]);
+      const float l2 = FORM == kFormFp32 ? log2f(v[u]) : lg2(v[u]);
+      al[i][u] = alpha;
+      t[i][u] = fmaf(fmaf(2.f * kap, mr, -kap * kap), a.c, l2);
+    }
+  }
+}
+
+// One unit by the tilted product.  False, with nothing written, when a sum left the range of FP32
+// (warp-uniform).
+template <int MODE, int FORM, int TN, bool PLAIN>
+__device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, float kc, const RowView& rv, int W, bool up,
+                                          const Tilt<FORM>& tilt, bool skip) {
+  f32x2 D[TN < 16 ? 1 : TN / 16][2];
+  window_product<FORM, TN, PLAIN>(a, kc, rv, W, up, tilt, D);
+  float al[TN < 16 ? 1 : TN / 8][2], t[TN < 16 ? 1 : TN / 8][2];   // (an empty row has sums 0: log -inf)
+  log_sums<FORM, TN>(a, kc, rv, !PLAIN && up ? walk_end(W) : 0, D, al, t);
+  return write_unit<MODE, TN>(a, r0, k0, al, t, skip);
+}
+
+// Exact window sum of one lane's output o of `row`, window [lo, lo + wl), xp[m] that row's position
+// m.  Terms are taken relative to e(mh, o), which is within the range of FP32 of the maximum unless
+// the maximum moves far from mh within the tile; a sum that overflows is done again from its exact
+// maximum.
 template <int MODE>
-__device__ __forceinline__ void exact_pair(const BandArgs& a, int row, int k0, int lo, int wl, int mh, const float* xp,
-                                           bool vec, bool skip) {
-  const int o = k0 + (threadIdx.x & 15);
+__device__ __forceinline__ void exact_output(const BandArgs& a, int row, int o, int lo, int wl, int mh, const float* xp,
+                                             bool vec, bool skip) {
   const float fo = (float)o + a.shift, sc = a.x_scale, nc = -a.c;
   float out = -INFINITY;
   if (wl > 0) {
@@ -504,97 +598,128 @@ __device__ __forceinline__ void exact_pair(const BandArgs& a, int row, int k0, i
   if (bad) raise_error(a.err, FOT_ENONFINITE);
 }
 
-// the rows of a unit outside the tilted product, two at a time
-template <int MODE>
-__device__ __forceinline__ void exact_unit(const BandArgs& a, int r0, int k0, RowView rv, bool skip) {
-  const int half = (threadIdx.x & 31) >> 4;
-  for (int p = 0; p < 4; ++p) {
-    const int src = 4 * (2 * p + half);
-    const int l = __shfl_sync(0xffffffffu, rv.lo, src), w = __shfl_sync(0xffffffffu, rv.wl, src);
-    const int m = __shfl_sync(0xffffffffu, rv.mh, src);
-    const float* xr = (const float*)__shfl_sync(0xffffffffu, (unsigned long long)rv.row, src);
-    exact_pair<MODE>(a, r0 + 2 * p + half, k0, l, w, m, xr, rv.vec, skip);
-  }
+// How a unit's rows stay in range of the tilted product (the top): 0 walking down, 1 walking up,
+// 2 not at all (warp-uniform)
+__device__ __forceinline__ int unit_walk(float kmax, const RowView& rv, int W, float c) {
+  const float t = 2.f * kmax * c, far = t * (float)max(rv.mh - rv.lo, rv.lo + rv.wl - rv.mh);
+  const bool none = rv.wl == 0, in = far <= kTiltMax;
+  if (__all_sync(0xffffffffu, none || (in && far + t * (float)(rv.mh - rv.lo) <= kRangeMax))) return 0;
+  return __all_sync(0xffffffffu, none || (in && far + t * (float)abs(rv.lo + walk_end(W) - rv.mh) <= kRangeMax)) ? 1 : 2;
 }
 
-// whether a row's operands stay in range of the tilted product (the top)
-__device__ __forceinline__ bool row_in_range(float kmax, int lo, int hi, int mh, float c) {
-  const float t = 2.f * kmax * c, far = t * (float)max(mh - lo, hi - mh);
-  return far <= kTiltMax && far + t * (float)(mh - lo) <= kRangeMax;
-}
-
-// a 32-wide unit outside the bound: two 16-wide ones with the rows' exact maxima at their own
-// centres, over the same windows (which cover theirs)
-template <int MODE, int FORM>
-__device__ __forceinline__ void split_unit(const BandArgs& a, int r0, int k0, RowView rv, int W, bool skip,
-                                        unsigned long long* terms) {
-  const int lane = threadIdx.x & 31, q = lane & 3;
+// every row's exact maximum over its window at centre kc, and where it is reached
+__device__ __forceinline__ RowView recentred(const BandArgs& a, const RowView& rv, float kc) {
+  const int q = threadIdx.x & 3;
   const float c = a.c, sc = a.x_scale;
-  for (int sub = 0; sub < 2; ++sub) {
-    const int ks = k0 + 16 * sub;
-    if (ks >= a.n_out) break;
-    const float kc = (float)(ks + 8) + a.shift;
-    RowView r = rv;
-    r.alpha = -INFINITY;
-    for (int p = 4 * q; p < rv.wl; p += 16) {
-      const float4 x = fetch4(rv.row, rv.lo + p, rv.wl - p, rv.vec);
-      const float xs[4] = {x.x, x.y, x.z, x.w};
+  RowView r = rv;
+  r.alpha = -INFINITY;
+  for (int p = 4 * q; p < rv.wl; p += 16) {
+    const float4 x = fetch4(rv.row, rv.lo + p, rv.wl - p, rv.vec);
+    const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float d = kc - (float)(rv.lo + p + u);
-        const float e = fmaf(-d * d, c, xs[u] * sc);
-        if (e > r.alpha) {
-          r.alpha = e;
-          r.mh = rv.lo + p + u;
-        }
+    for (int u = 0; u < 4; ++u) {
+      const float d = kc - (float)(rv.lo + p + u);
+      const float e = fmaf(-d * d, c, xs[u] * sc);
+      if (e > r.alpha) {
+        r.alpha = e;
+        r.mh = rv.lo + p + u;
       }
     }
-#pragma unroll
-    for (int d = 1; d < 4; d <<= 1) {
-      const float oa = __shfl_xor_sync(0xffffffffu, r.alpha, d);
-      const int om = __shfl_xor_sync(0xffffffffu, r.mh, d);
-      if (oa > r.alpha || (oa == r.alpha && om < r.mh)) {
-        r.alpha = oa;
-        r.mh = om;
-      }
-    }
-    if (__all_sync(0xffffffffu, r.wl == 0 || row_in_range(8.f, r.lo, r.lo + r.wl, r.mh, c))) {
-      if (lane == 0) atomicAdd(terms + (FORM == kFormFp32 ? 0 : 2), (unsigned long long)W * 16 * 8);
-      Tilt<FORM> tilt;
-      tilt.load(a, 16, false);
-      if (gemm_unit<MODE, FORM, 16, false>(a, r0, ks, kc, r, W, tilt, skip)) continue;
-    }
-    if (q == 0) atomicAdd(terms + 1, (unsigned long long)r.wl * 16);
-    exact_unit<MODE>(a, r0, ks, r, skip);
   }
+#pragma unroll
+  for (int d = 1; d < 4; d <<= 1) {
+    const float oa = __shfl_xor_sync(0xffffffffu, r.alpha, d);
+    const int om = __shfl_xor_sync(0xffffffffu, r.mh, d);
+    if (oa > r.alpha || (oa == r.alpha && om < r.mh)) {
+      r.alpha = oa;
+      r.mh = om;
+    }
+  }
+  return r;
 }
 
-// a unit whose rows are not staged, or that is outside the bound, or whose sums left the range of
-// FP32 (try_product false)
-template <int MODE, int FORM>
-__device__ __noinline__ void other_unit(const BandArgs& a, int r0, int k0, RowView rv, int W, bool try_product, bool skip,
-                                        unsigned long long* terms) {
-  if (try_product) {
+// A unit outside the bound, in segments of its window (the top).  False, with nothing written, when
+// it cannot be done that way (warp-uniform).
+template <int MODE, int TN>
+__device__ __noinline__ bool segmented_unit(const BandArgs& a, int r0, int k0, const RowView& rv, int W, bool skip,
+                                            unsigned long long* terms) {
+  constexpr int NO = TN < 16 ? 1 : TN / 8;
+  const float kc = (float)(k0 + TN / 2) + a.shift, c = a.c;
+  const int L = min((int)(kRangeMax / (2.f * TN * c)) & ~15, 4096);   // TN (D + mh - lo) c <= TN 2 L c
+  if (L < 16) return false;
+  Tilt<kFormFp32> tilt;
+  tilt.load(a, TN, false);
+  float A[NO][2], T[NO][2];                               // the sums so far: offset and rest
+#pragma unroll
+  for (int i = 0; i < NO; ++i)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      A[i][u] = -INFINITY;
+      T[i][u] = 0.f;
+    }
+  for (int s0 = 0; s0 < W; s0 += L) {
+    RowView r = rv;
+    r.lo = rv.lo + s0;
+    r.wl = max(0, min(rv.wl - s0, L));
+    r = recentred(a, r, kc);
+    if (r.alpha == -INFINITY) r.wl = 0;
+    // against mh's term, a term m of the segment gains at most TN |m - mh| c at the tile's ends
+    const float gain = (float)TN * c * (float)max(abs(r.lo - rv.mh), abs(r.lo + r.wl - rv.mh));
+    if (!__any_sync(0xffffffffu, r.wl > 0 && r.alpha + gain >= rv.alpha - kCut)) continue;
+    const int Ws = __reduce_max_sync(0xffffffffu, r.wl);
+    if ((threadIdx.x & 31) == 0) atomicAdd(terms, (unsigned long long)Ws * TN * 8);
+    f32x2 D[TN < 16 ? 1 : TN / 16][2];
+    window_product<kFormFp32, TN, false>(a, kc, r, Ws, false, tilt, D);
+    float al[NO][2], t[NO][2];
+    log_sums<kFormFp32, TN>(a, kc, r, 0, D, al, t);
+#pragma unroll
+    for (int i = 0; i < NO; ++i)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        // (A, T) <- log2(2^(A + T) + 2^(al + t)); the offsets are subtracted first
+        if (al[i][u] == -INFINITY) continue;
+        const float d = (al[i][u] - A[i][u]) + (t[i][u] - T[i][u]);
+        const bool up = !(d < 0.f);                       // the new one is the larger (or the first)
+        const float more = log2f(1.f + ex2(up ? -d : d));
+        A[i][u] = up ? al[i][u] : A[i][u];
+        T[i][u] = (up ? t[i][u] : T[i][u]) + more;
+      }
+  }
+  return write_unit<MODE, TN>(a, r0, k0, A, T, skip);
+}
+
+// a unit that is not the common case: a narrow tile, rows not staged, a long window, walking up,
+// outside the bound or with sums that left the range of FP32 (walk 2: no product)
+template <int MODE, int FORM, int TN>
+__device__ __forceinline__ void other_unit_of(const BandArgs& a, int r0, int k0, const RowView& rv, int W, int walk,
+                                              bool skip, unsigned long long* terms) {
+  if (walk != 2) {
     Tilt<FORM> tilt;
-    tilt.load(a, a.tile_w, true);
-    const float kc = (float)(k0 + (a.tile_w >> 1)) + a.shift;
-    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, false>(a, r0, k0, kc, rv, W, tilt, skip)
-                       : gemm_unit<MODE, FORM, 16, false>(a, r0, k0, kc, rv, W, tilt, skip))
-      return;
+    tilt.load(a, TN, TN >= 16);
+    if (gemm_unit<MODE, FORM, TN, false>(a, r0, k0, (float)(k0 + TN / 2) + a.shift, rv, W, walk == 1, tilt, skip)) return;
   }
-  if (a.tile_w == 32) {
-    split_unit<MODE, FORM>(a, r0, k0, rv, W, skip, terms);
-  } else {
-    if ((threadIdx.x & 3) == 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
-    exact_unit<MODE>(a, r0, k0, rv, skip);
-  }
+  if (segmented_unit<MODE, TN>(a, r0, k0, rv, W, skip, terms)) return;
+  const int lane = threadIdx.x & 31;
+  if ((lane & 3) == 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * TN);
+  for (int k = k0; k < k0 + TN; k += 4)
+    exact_output<MODE>(a, r0 + (lane >> 2), k + (lane & 3), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, skip);
+}
+template <int MODE, int FORM>
+__device__ __noinline__ void other_unit(const BandArgs& a, int r0, int k0, RowView rv, int W, int walk, bool skip,
+                                        unsigned long long* terms) {
+  if (a.tile_w == 32)
+    other_unit_of<MODE, FORM, 32>(a, r0, k0, rv, W, walk, skip, terms);
+  else if (a.tile_w == 16)
+    other_unit_of<MODE, FORM, 16>(a, r0, k0, rv, W, walk, skip, terms);
+  else
+    other_unit_of<MODE, kFormFp32, 8>(a, r0, k0, rv, W, walk, skip, terms);
 }
 
 // A warp's unit of the item that its CTA was launched for.
 struct Unit {
   RowView rv;
   int r0, k0, row;                                        // first row and output, this lane's row
-  bool pairs, out_of_range, skip;
+  bool pairs, skip;
 };
 
 // The start of a window CTA: read the item and this warp's plan entries, stage the rows; `meanwhile`
@@ -661,8 +786,7 @@ __device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const Band
   meanwhile();
   rv.lo = w1 & 0xffff;
   rv.wl = w1 >> 16;
-  rv.mh = w2 & 0xffff;
-  u.out_of_range = (w2 >> 16) != 0;
+  rv.mh = w2;
   rv.staged = staged;
   rv.vec = staged || (a.vec & 1);
   rv.row = staged ? rows + lr * pitch - base : a.x + (size_t)min(u.row, a.n_rows - 1) * a.len;
@@ -681,6 +805,23 @@ __device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const Band
   return __all_sync(0xffffffffu, ok) && tile < a.n_tiles;
 }
 
+// A pass whose problems all take exact sums: 2 rows x 16 outputs per warp.  Its own kernel for its
+// registers (12 CTAs per SM; inside the window kernel, with 4 or 5, a pass at 512^2 and eps 2 took
+// 25 us).
+template <int MODE, int MAXP>
+__global__ void __launch_bounds__(kWinThreads, 12) exact_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
+  extern __shared__ __align__(128) float s_x[];
+  __shared__ __align__(8) uint64_t s_bar;
+  const int lane = threadIdx.x & 31;
+  const BandArgs& a = tab.p[find_prob<MAXP, 1>(tab, (int)blockIdx.x)];
+  Unit u;
+  if (!open_unit(tab, a, s_x, &s_bar, u, []() {})) return;
+  const RowView& rv = u.rv;
+  if ((lane & 15) == 0 && rv.wl > 0)
+    atomicAdd(a.terms + 4 * (blockIdx.x & (kTermSlots - 1)) + 1, (unsigned long long)rv.wl * 16);
+  exact_output<MODE>(a, u.row, u.k0 + (lane & 15), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
+}
+
 template <int MODE, int FORM, int MAXP>
 __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
   extern __shared__ __align__(128) float s_x[];
@@ -690,28 +831,28 @@ __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window
   Unit u;
   Tilt<FORM> tilt;
   if (!open_unit(tab, a, s_x, &s_bar, u, [&]() {
-        if (a.group != 2) tilt.load(a, a.tile_w, true);
+        if (a.tile_w >= 16 && a.group != 2) tilt.load(a, a.tile_w, true);
       }))
     return;
   unsigned long long* terms = a.terms + 4 * (blockIdx.x & (kTermSlots - 1));
   const RowView& rv = u.rv;
   if (u.pairs) {
     if ((lane & 15) == 0 && rv.wl > 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
-    exact_pair<MODE>(a, u.row, u.k0, rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
+    exact_output<MODE>(a, u.row, u.k0 + (lane & 15), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
     return;
   }
   const int W = __reduce_max_sync(0xffffffffu, rv.wl);
-  const bool in_range = !__any_sync(0xffffffffu, u.out_of_range);
-  if (in_range && lane == 0 && W > 0)
-    atomicAdd(terms + (FORM == kFormFp32 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
-  const bool here = in_range && (rv.staged || W == 0);
-  if (here) {
+  const int walk = unit_walk(0.5f * (float)a.tile_w, rv, W, a.c);
+  if (walk != 2 && lane == 0 && W > 0)
+    atomicAdd(terms + (FORM == kFormFp32 || a.tile_w < 16 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
+  const bool plain = walk == 0 && a.tile_w >= 16 && (rv.staged || W == 0) && !long_window(W, a.c);
+  if (plain) {
     const float kc = (float)(u.k0 + (a.tile_w >> 1)) + a.shift;
-    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, tilt, u.skip)
-                       : gemm_unit<MODE, FORM, 16, true>(a, u.r0, u.k0, kc, rv, W, tilt, u.skip))
+    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip)
+                       : gemm_unit<MODE, FORM, 16, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip))
       return;
   }
-  other_unit<MODE, FORM>(a, u.r0, u.k0, rv, W, in_range && !here, u.skip, terms);
+  other_unit<MODE, FORM>(a, u.r0, u.k0, rv, W, plain ? 2 : walk, u.skip, terms);
 }
 
 // launch with programmatic dependence on the kernel before it in the stream: its set-up (and
@@ -732,9 +873,11 @@ void launch_dependent(K kernel, dim3 grid, int threads, size_t smem, cudaStream_
 }
 
 // dynamic shared memory of the window kernel: four -inf, eight rows (within the default 48 KB)
-__host__ __device__ inline size_t window_smem(int pitch) { return (size_t)(16 + 8 * pitch) * sizeof(float); }
+__host__ __device__ inline size_t window_smem(int pitch, int rows = 8) { return (size_t)(16 + rows * pitch) * sizeof(float); }
 
 template <int MODE, int FORM, int MAXP>
 void window_launch(cudaStream_t s, const BandTable<MAXP>& t);
+template <int MODE, int MAXP>
+void exact_launch(cudaStream_t s, const BandTable<MAXP>& t);
 
 }  // namespace fot
