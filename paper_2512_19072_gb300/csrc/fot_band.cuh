@@ -105,6 +105,17 @@ void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form);
 template <int MAXP>
 void plan_pass(cudaStream_t s, BandTable<MAXP>& t);
 
+// words of the window plan and items of the window kernel for a context's passes
+inline size_t band_plan_words(int rows, int cols) {
+  const size_t pr = (size_t)(rows + 7) / 8 * 8, pc = (size_t)(cols + 7) / 8 * 8;
+  const size_t a = pr * plan_tiles(cols), b = pc * plan_tiles(rows);
+  return 3 * (a > b ? a : b);
+}
+inline size_t band_items(int rows, int cols) {
+  const size_t a = (size_t)(rows + 7) / 8 * ((plan_tiles(cols) + 3) / 4), b = (size_t)(cols + 7) / 8 * ((plan_tiles(rows) + 3) / 4);
+  return a > b ? a : b;
+}
+
 int form_of(const fot_ctx* c);
 
 constexpr int kTiltTables = 256;   // tilt tables a context holds

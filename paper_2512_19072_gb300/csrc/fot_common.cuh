@@ -65,6 +65,7 @@ void ktimer_end(cudaStream_t s);
 struct fot_ctx {
   int rows = 0, cols = 0, device = 0, precision = 0;
   cudaStream_t stream = nullptr;
+  unsigned char* mem = nullptr;   // the allocation that holds every buffer below unless noted
   // device images, rows x cols unless noted
   float* la = nullptr;       // log a (natural), -inf on zero mass
   float* lb = nullptr;       // log b
