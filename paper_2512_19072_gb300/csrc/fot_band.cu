@@ -354,6 +354,7 @@ void plan_pass(cudaStream_t s, BandTable<MAXP>& t) {
 }
 
 template void plan_pass<1>(cudaStream_t, BandTable<1>&);
+template void plan_pass<2>(cudaStream_t, BandTable<2>&);
 template void plan_pass<kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&);
 
 template <int MODE, int MAXP>
@@ -375,6 +376,8 @@ void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
 
 template void band_pass<0, 1>(cudaStream_t, BandTable<1>&, int);
 template void band_pass<1, 1>(cudaStream_t, BandTable<1>&, int);
+template void band_pass<0, 2>(cudaStream_t, BandTable<2>&, int);
+template void band_pass<1, 2>(cudaStream_t, BandTable<2>&, int);
 template void band_pass<0, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
 template void band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
 
@@ -382,6 +385,8 @@ template void band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
 cudaError_t plan_configure() {
   const int lim = (int)(kPlanRows * plan_row_floats(4096 / kCW) * sizeof(float)) + 2 * 256 * (int)sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(band_plan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(band_plan_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(band_plan_kernel<kMaxBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   return e;
@@ -474,6 +479,42 @@ void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double 
   t.p[0].lmarg = lmarg;
   t.p[0].logsum = logsum;
   band_pass<1>(c->stream, t, form);
+  c->launches += k;
+}
+
+// Two half-steps of one context in the same launches (2 per pass).
+void half_step_band_pair(fot_ctx* c, const float* inA, const float* inB, const float* lmarg, double eps, float* outA,
+                         float* outB, float* logsumA, float* logsumB, const PairSpace& second) {
+  const int form = form_of(c);
+  BandTable<2> t{};
+  t.n = 2;
+  t.spin_limit = c->spin;
+  int64_t k = 2 * 2;
+  const uint4* tilt = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int q = 0; q < 2; ++q) {
+      BandArgs& a = t.p[q];
+      float* R = q == 0 ? c->R : second.R;
+      a = pass == 0 ? band_args(c, q == 0 ? inA : inB, c->rows, c->cols, eps, (float)(1.4426950408889634 / eps))
+                    : band_args(c, R, c->cols, c->rows, eps, 1.f);
+      if (pass == 0 && q == 0) tilt = tilt_for(c, eps, a.group == 8 ? a.tile_w : 0, &k);
+      a.tilt = tilt;
+      if (q == 1) {
+        a.plan = second.plan;
+        a.items = second.items;
+        a.order = second.order;
+      }
+      a.y = pass == 0 ? R : q == 0 ? outA : outB;
+      if (pass == 1) {
+        a.lmarg = lmarg;
+        a.logsum = q == 0 ? logsumA : logsumB;
+      }
+    }
+    if (pass == 0)
+      band_pass<0>(c->stream, t, form);
+    else
+      band_pass<1>(c->stream, t, form);
+  }
   c->launches += k;
 }
 

@@ -105,6 +105,17 @@ void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form);
 template <int MAXP>
 void plan_pass(cudaStream_t s, BandTable<MAXP>& t);
 
+// work space of the second problem of a two-problem pass
+struct PairSpace {
+  float* plan;
+  int4* items;
+  int* order;          // zeroed before the first use
+  float* R;
+};
+// logsums of two inputs of a context's half-step in two-problem passes (outA, outB: potentials)
+void half_step_band_pair(fot_ctx* c, const float* inA, const float* inB, const float* lmarg, double eps, float* outA,
+                         float* outB, float* logsumA, float* logsumB, const PairSpace& second);
+
 // words of the window plan and items of the window kernel for a context's passes
 inline size_t band_plan_words(int rows, int cols) {
   const size_t pr = (size_t)(rows + 7) / 8 * 8, pc = (size_t)(cols + 7) / 8 * 8;

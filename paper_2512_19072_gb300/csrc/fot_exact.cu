@@ -10,6 +10,8 @@ void exact_launch(cudaStream_t s, const BandTable<MAXP>& t) {
 
 template void exact_launch<0, 1>(cudaStream_t, const BandTable<1>&);
 template void exact_launch<1, 1>(cudaStream_t, const BandTable<1>&);
+template void exact_launch<0, 2>(cudaStream_t, const BandTable<2>&);
+template void exact_launch<1, 2>(cudaStream_t, const BandTable<2>&);
 template void exact_launch<0, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 template void exact_launch<1, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 

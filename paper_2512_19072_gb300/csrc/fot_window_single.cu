@@ -11,6 +11,8 @@ void window_launch(cudaStream_t s, const BandTable<MAXP>& t) {
 
 template void window_launch<0, kFormSingle, 1>(cudaStream_t, const BandTable<1>&);
 template void window_launch<1, kFormSingle, 1>(cudaStream_t, const BandTable<1>&);
+template void window_launch<0, kFormSingle, 2>(cudaStream_t, const BandTable<2>&);
+template void window_launch<1, kFormSingle, 2>(cudaStream_t, const BandTable<2>&);
 template void window_launch<0, kFormSingle, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 template void window_launch<1, kFormSingle, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 

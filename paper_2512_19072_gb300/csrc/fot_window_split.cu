@@ -11,6 +11,8 @@ void window_launch(cudaStream_t s, const BandTable<MAXP>& t) {
 
 template void window_launch<0, kFormSplit, 1>(cudaStream_t, const BandTable<1>&);
 template void window_launch<1, kFormSplit, 1>(cudaStream_t, const BandTable<1>&);
+template void window_launch<0, kFormSplit, 2>(cudaStream_t, const BandTable<2>&);
+template void window_launch<1, kFormSplit, 2>(cudaStream_t, const BandTable<2>&);
 template void window_launch<0, kFormSplit, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 template void window_launch<1, kFormSplit, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 

@@ -147,3 +147,29 @@ def test_adjoint_backward_workload_directional_fd(fot_lib):
                 ad = float((grad * v).sum())
                 assert abs(fd - ad) <= 2e-2 * abs(ad), (which, kind, fd, ad)
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "mixed", "fp32_dense"])
+@pytest.mark.parametrize("rows,cols,every", [(1, 300, 1), (300, 1, 3), (2, 2, 7), (5, 261, 2), (67, 9, 2)])
+def test_adjoint_lines_and_segments(fot_lib, prec, rows, cols, every):
+    """Lines of one chunk and of several, single rows and columns, segments of one iteration, a
+    remainder and more than all iterations.  Bound: the exponents of the weights reach
+    C/eps = 300^2 / (2 * 60) = 750, so one FP32 rounding of an exponent is 4.5e-5 relative; ten
+    such in a row (5 iterations, two half-steps each) stay below 2e-3 of the largest entry."""
+    B = fot_lib
+    P = {"fp32": B.FOT_FP32, "mixed": B.FOT_MIXED, "fp32_dense": B.FOT_FP32_DENSE}[prec]
+    rng = np.random.default_rng(46)
+    g = f32(rng.uniform(0.3, 1.0, size=(rows, cols)))
+    G = f32(rng.uniform(0.3, 1.0, size=(rows, cols)))
+    w = f32(rng.uniform(0, 1, size=(rows, cols)))
+    phi_t = f32(rng.normal(0, 0.1, size=(rows, cols)))
+    dx = 0.1
+    _, dg_ref, dG_ref = adjoint.gradients(g, G, 60.0, 5, w, phi_t, dx)
+    gt, Gt = to_dev(g), to_dev(G)
+    ctx = B.fot_create(rows, cols, P)
+    B.fot_solve(ctx, gt, Gt, [60.0], 5, dx=dx)
+    phi, _, _ = B.fot_phase(ctx)
+    dg, dG = B.fot_backward(ctx, gt, Gt, dL_dphi=_loss_seed(phi, to_dev(w), to_dev(phi_t)), checkpoint_every=every)
+    for got, ref in ((dg.double().cpu().numpy(), dg_ref), (dG.double().cpu().numpy(), dG_ref)):
+        assert np.abs(got - ref).max() <= 2e-3 * np.abs(ref).max(), np.abs(got - ref).max() / np.abs(ref).max()
+    ctx.close()
