@@ -349,8 +349,8 @@ fot_status fot_work_split(fot_ctx* ctx, int64_t* out4);
 
 /* Kernel classes of fot_kernel_times. */
 enum {
-  FOT_KERNEL_PLAN = 0,     /* window plan of a banded pass (and the tilt tables of the BF16 forms,
-                              written once per loop) */
+  FOT_KERNEL_PLAN = 0,     /* window plan of a banded pass, whole passes whose plan and sums are one
+                              kernel (exact sums, small problems), tilt tables of the BF16 forms */
   FOT_KERNEL_BAND = 1,     /* window sums of a banded pass, FP32 operands */
   FOT_KERNEL_TENSOR = 2,   /* window sums of a banded pass, BF16 operands */
   FOT_KERNEL_DENSE = 3,    /* dense exact pass */

@@ -34,7 +34,7 @@ void c_transform_envelope(fot_ctx* c, const float* pot_in, float* out);
 void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double eps,
                     float* pot_out, float* logsum);
 size_t tilt_bytes();
-cudaError_t plan_configure();
+cudaError_t plan_configure(int longest);
 int default_wait_limit();
 }  // namespace fot
 
@@ -195,7 +195,7 @@ fot_status fot_create(fot_ctx** out, int rows, int cols, int precision, int devi
     ok = cudaMemsetAsync(c->mem + at_zero, 0, need - at_zero, c->stream) == cudaSuccess;
   }
   if (ok) ok = cudaEventCreate(&c->ev_loop0) == cudaSuccess && cudaEventCreate(&c->ev_loop1) == cudaSuccess;
-  if (ok && (simt_configure() != cudaSuccess || plan_configure() != cudaSuccess)) {   // per-device kernel attributes
+  if (ok && (simt_configure() != cudaSuccess || plan_configure(rows > cols ? rows : cols) != cudaSuccess)) {   // per-device kernel attributes
     cudaGetLastError();
     fot_destroy(c);
     return FOT_ECUDA;

@@ -1,30 +1,10 @@
 // Banded axis passes: the same contraction as the exact pass,
 //     y[o][r] = log2 sum_m 2^( x[r][m]*scale - (o - m)^2 c ),   c = log2(e) / (2 eps),
 // but each output only visits the terms that can matter, and where eps allows the inner sum is
-// a matrix product instead of one exponential per term.  A pass is two kernels: the window plan
-// (this file) and the window sums (fot_window.cuh, which describes the arithmetic).
-//
-// The plan leaves, per (row, tile of tile_w outputs), an offset alpha, the position mh it was
-// taken at and a window [lo, lo + wl):
-//
-// 1. alpha = e(mh, kc), e(m, o) = x[m] scale - (o - m)^2 c, at the tile centre kc: the maximum
-//    over the 32-wide chunk whose own maximum gives the best term there.  It may lie below the
-//    exact maximum, which only raises the operands 2^(e - alpha) of the window sums (a sum that
-//    leaves the range of FP32 is done again there).
-// 2. A provable window: every o in the tile has max_m e(m, o) >= LB = min over the tile's two
-//    ends of e(mh, o) (e(mh, .) is concave).  A block of 8 positions whose bound (its maximum
-//    at its nearest distance to the tile) lies below LB - kCut holds only terms below 2^-kCut
-//    of every output of the tile; the window is the hull of the remaining blocks (found per
-//    32-wide chunk first, then narrowed from both ends).
-// Arg-maxima carry the index in the low mantissa bits of the value they compare (5 bits for a
-// position, 7 for a chunk): one maximum instead of a compare and two selects; a chunk's maximum
-// is rounded by 2^-18 of itself that way, far inside the margin of kCut.
-//
-// What bounds it: latency and issue slots (4 MB of input at 1024^2, in L2).  Two lanes serve a
-// (row, tile): each takes every other pair of chunks (packed FP32 pairs), half of the scanned
-// chunk and one end of the window.  Chunks are padded to 36 words: lanes on different chunks read
-// different banks, lanes on the same chunk broadcast.
-#include "fot_window.cuh"
+// a matrix product instead of one exponential per term.  A pass is two kernels, the window plan
+// (fot_plan.cuh) and the window sums (fot_window.cuh, which describes the arithmetic), or one that does
+// both (fot_small.cuh).  This file has the plan's kernel and chooses between them.
+#include "fot_small.cuh"
 
 #include <math.h>
 
@@ -34,40 +14,18 @@ namespace fot {
 
 namespace {
 
-constexpr int kPlanRows = 8;                  // rows of a CTA: one row group of the window kernel
-constexpr int kPlanThreads = 512;
-constexpr int kPlanQ = 2;                     // lanes per (row, tile)
-constexpr int kZS = kCW + 4;                  // words of a staged chunk
-
-// shared memory of one row (floats): chunk maxima and minus their positions (rounded up to four
-// chunks each), block maxima [n_chunks * 4], z [n_chunks * kZS]
-__host__ __device__ inline int plan_row_floats(int n_chunks) { return 2 * ((n_chunks + 3) & ~3) + n_chunks * (4 + kZS); }
-
-// v with its low mantissa bits replaced by an index (-inf becomes a NaN, which fmaxf drops)
-template <int BITS>
-__device__ __forceinline__ float tagged(float v, int index) {
-  return __uint_as_float((__float_as_uint(v) & ~((1u << BITS) - 1u)) | (uint32_t)index);
-}
-template <int BITS>
-__device__ __forceinline__ int tag_of(float v) { return (int)(__float_as_uint(v) & ((1u << BITS) - 1u)); }
-
 template <int MAXP>
 __global__ void __launch_bounds__(kPlanThreads) band_plan_kernel(const __grid_constant__ BandTable<MAXP> tab) {
   extern __shared__ __align__(16) float s_plan[];
   const int tid = threadIdx.x;
   const BandArgs& a = tab.p[find_prob<MAXP, 0>(tab, (int)blockIdx.x)];
   const int rg = (int)blockIdx.x - a.plan_base;           // row group of the problem
-  const int T = a.n_tiles, len = a.len, nch = a.n_chunks, tw = a.tile_w;
-  const float c = a.c, sc = a.x_scale;
+  const int T = a.n_tiles;
   // threads per row: a power of two (at least kPlanQ lanes of one warp serve a (row, tile))
   const int tpr = 1 << tab.plan_tpr_log2, rr = tid >> tab.plan_tpr_log2, ti = tid & (tpr - 1);
   const int row = kPlanRows * rg + rr;
   const bool live = row < a.n_rows;
-  float* const cm = s_plan + (size_t)rr * tab.plan_row_floats;
-  const int nchp = (nch + 3) & ~3;
-  float* const np_ = cm + nchp;                           // minus the maxima's positions
-  float* const bm = np_ + nchp;
-  float* const z = bm + 4 * nch;
+  float* const mine = s_plan + (size_t)rr * tab.plan_row_floats;
   // per item (four tiles): the span of its windows
   int* const s_lo = reinterpret_cast<int*>(s_plan + (size_t)kPlanRows * tab.plan_row_floats);
   int* const s_hi = s_lo + tab.plan_items;
@@ -78,173 +36,36 @@ __global__ void __launch_bounds__(kPlanThreads) band_plan_kernel(const __grid_co
   grid_wait();
   grid_launch_next();
 
-  // ---- stage: blocks of 8 positions, a thread each; four neighbouring threads share a chunk
-  {
-    const float* xr = a.x + (size_t)row * len;
-    const bool vec = (a.vec & 1) != 0;
-    const f32x2 sc2 = pack2(sc, sc);
-    for (int b = ti; b < nchp * 4; b += tpr) {
-      const int m0 = b * 8, j = b >> 2, u0 = (b & 3) * 8;
-      float v[8];
-      if (live && vec && m0 + 8 <= len) {
-        const float4 p = __ldg(reinterpret_cast<const float4*>(xr + m0)), q = __ldg(reinterpret_cast<const float4*>(xr + m0) + 1);
-        v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
-        v[4] = q.x; v[5] = q.y; v[6] = q.z; v[7] = q.w;
-      } else {
+  const float* const xr = a.x + (size_t)row * a.len;
+  plan_stage(a, mine, ti, tpr, [&](int m0, float (&v)[8]) {
+    if (live && (a.vec & 1) && m0 + 8 <= a.len) {
+      const float4 p = __ldg(reinterpret_cast<const float4*>(xr + m0)), q = __ldg(reinterpret_cast<const float4*>(xr + m0) + 1);
+      v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
+      v[4] = q.x; v[5] = q.y; v[6] = q.z; v[7] = q.w;
+    } else {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = live && m0 + u < len ? __ldg(xr + m0 + u) : -INFINITY;
-      }
-      float best = -INFINITY, top = -INFINITY;            // block maximum; the same with its position
-#pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        unpack2(mul2(pack2(v[u], v[u + 1]), sc2), v[u], v[u + 1]);
-        best = fmaxf(best, fmaxf(v[u], v[u + 1]));
-        top = fmaxf(top, fmaxf(tagged<5>(v[u], u0 + u), tagged<5>(v[u + 1], u0 + u + 1)));
-      }
-      if (j < nch) {
-        float4* const zb = reinterpret_cast<float4*>(z + j * kZS + u0);
-        zb[0] = make_float4(v[0], v[1], v[2], v[3]);
-        zb[1] = make_float4(v[4], v[5], v[6], v[7]);
-        bm[b] = best;
-      }
-      // (the four threads of a chunk are neighbours and take this iteration together)
-      const unsigned quad = 0xfu << (tid & 28);
-      top = fmaxf(top, __shfl_xor_sync(quad, top, 1));
-      top = fmaxf(top, __shfl_xor_sync(quad, top, 2));
-      best = fmaxf(best, __shfl_xor_sync(quad, best, 1));
-      best = fmaxf(best, __shfl_xor_sync(quad, best, 2));
-      if (u0 == 0) {
-        cm[j] = best;
-        np_[j] = -(float)(j * kCW + tag_of<5>(top));
-      }
+      for (int u = 0; u < 8; ++u) v[u] = live && m0 + u < a.len ? __ldg(xr + m0 + u) : -INFINITY;
     }
-  }
+  });
   __syncthreads();
 
-  // ---- kPlanQ lanes per (row, tile)
+  // kPlanQ lanes per (row, tile)
   const size_t np = (size_t)a.plan_stride * T;
   int* const plan_i = reinterpret_cast<int*>(a.plan);
   const int q = ti & (kPlanQ - 1);
-  const f32x2 nc2 = pack2(-c, -c);
-  // (lanes past the tiles or rows compute on a valid place and write nothing: the shuffles below
-  // want whole warps)
+  // (lanes past the tiles or rows compute on a valid place and write nothing: the shuffles want
+  // whole warps)
   for (int t0 = 0; t0 < T; t0 += tpr / kPlanQ) {
     const int t = min(t0 + ti / kPlanQ, T - 1);
-    const bool has = live && t0 + ti / kPlanQ < T;
-    const float f0 = (float)(t * tw) + a.shift;            // the tile's ends and centre
-    const float f1 = (float)(min((t + 1) * tw, a.n_out) - 1) + a.shift;
-    const float fkc = (float)(t * tw + tw / 2) + a.shift;
-
-    // the chunk whose maximum gives the best term at kc
-    float vb = -INFINITY;
-    const f32x2 kc2 = pack2(fkc, fkc);
-#pragma unroll 4
-    for (int j = 2 * q; j < nchp; j += 2 * kPlanQ) {
-      const float2 m = *reinterpret_cast<const float2*>(cm + j), p = *reinterpret_cast<const float2*>(np_ + j);
-      const f32x2 d = add2(kc2, pack2(p.x, p.y));
-      float v0, v1;
-      unpack2(fma2(mul2(d, d), nc2, pack2(m.x, m.y)), v0, v1);
-      vb = fmaxf(vb, fmaxf(tagged<7>(v0, j), tagged<7>(v1, j + 1)));
-    }
-#pragma unroll
-    for (int d = 1; d < kPlanQ; d <<= 1) vb = fmaxf(vb, __shfl_xor_sync(0xffffffffu, vb, d));
-    const bool any = vb != -INFINITY;                     // some term is finite
-    const int jb = any ? tag_of<7>(vb) : 0;
-
-    // the maximum over that chunk (half of it for each lane)
-    float sb = -INFINITY;
-    {
-      constexpr int kShare = kCW / kPlanQ;
-      const float* zj = z + jb * kZS + q * kShare;
-      const float d0 = fkc - (float)(jb * kCW + q * kShare);
-      f32x2 d01 = pack2(d0, d0 - 1.f);
-      const f32x2 dn2 = pack2(-2.f, -2.f);
-#pragma unroll
-      for (int u = 0; u < kShare; u += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(zj + u);
-        float v0, v1, v2, v3;
-        unpack2(fma2(mul2(d01, d01), nc2, pack2(x.x, x.y)), v0, v1);
-        d01 = add2(d01, dn2);
-        unpack2(fma2(mul2(d01, d01), nc2, pack2(x.z, x.w)), v2, v3);
-        d01 = add2(d01, dn2);
-        const int i = q * kShare + u;
-        sb = fmaxf(sb, fmaxf(tagged<5>(v0, i), tagged<5>(v1, i + 1)));
-        sb = fmaxf(sb, fmaxf(tagged<5>(v2, i + 2), tagged<5>(v3, i + 3)));
-      }
-    }
-#pragma unroll
-    for (int d = 1; d < kPlanQ; d <<= 1) sb = fmaxf(sb, __shfl_xor_sync(0xffffffffu, sb, d));
-    const int ub = tag_of<5>(sb);
-    const float zm = z[jb * kZS + ub];
-    int mh = jb * kCW + ub;
-    const float fm = (float)mh;
-    const float dk = fkc - fm, da = f0 - fm, db = f1 - fm;
-    const float alpha = fmaf(-dk * dk, c, zm);
-    const float lb = fminf(fmaf(-da * da, c, zm), fmaf(-db * db, c, zm)) - kCut;
-
-    // the window in chunks
-    int wlo = 0x7fffffff, whi = -1;
-    {
-      const float c0 = (float)(2 * q * kCW);
-      f32x2 e0 = pack2(f0 - c0 - (float)(kCW - 1), f0 - c0 - (float)(2 * kCW - 1));   // f0 - chunk's last
-      f32x2 e1 = pack2(c0 - f1, c0 + (float)kCW - f1);                                // chunk's first - f1
-      const f32x2 up = pack2((float)(2 * kPlanQ * kCW), (float)(2 * kPlanQ * kCW));
-      const f32x2 dn = pack2(-(float)(2 * kPlanQ * kCW), -(float)(2 * kPlanQ * kCW));
-#pragma unroll 4
-      for (int j = 2 * q; j < nchp; j += 2 * kPlanQ) {
-        const float2 m = *reinterpret_cast<const float2*>(cm + j);
-        float a0, a1, b0, b1, v0, v1;
-        unpack2(e0, a0, a1);
-        unpack2(e1, b0, b1);
-        const f32x2 d = pack2(fmaxf(fmaxf(a0, b0), 0.f), fmaxf(fmaxf(a1, b1), 0.f));
-        e0 = add2(e0, dn);
-        e1 = add2(e1, up);
-        unpack2(fma2(mul2(d, d), nc2, pack2(m.x, m.y)), v0, v1);
-        if (v0 >= lb) {
-          wlo = min(wlo, j);
-          whi = j;
-        }
-        if (v1 >= lb) {
-          wlo = min(wlo, j + 1);
-          whi = j + 1;
-        }
-      }
-    }
-#pragma unroll
-    for (int d = 1; d < kPlanQ; d <<= 1) {
-      wlo = min(wlo, __shfl_xor_sync(0xffffffffu, wlo, d));
-      whi = max(whi, __shfl_xor_sync(0xffffffffu, whi, d));
-    }
-    // narrow the hull block by block, chunk by chunk: lane 0 from its start, lane 1 from its end
-    // (it holds mh's block, whose bound reaches LB)
-    const bool win = any && whi >= 0;
-    int j = win ? (q == 0 ? wlo : whi) : 0, edge = 0;
-    const int jend = win ? (q == 0 ? whi : wlo) : 0, jstep = q == 0 ? 1 : -1;
-    for (;;) {
-      const float4 m = *reinterpret_cast<const float4*>(bm + 4 * j);
-      const float ms[4] = {m.x, m.y, m.z, m.w};
-      const float a0 = f0 - (float)(j * kCW) - 7.f, b0 = (float)(j * kCW) - f1;
-      int mask = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float d = fmaxf(fmaxf(a0 - 8.f * i, b0 + 8.f * i), 0.f);
-        if (fmaf(-d * d, c, ms[i]) >= lb) mask |= 1 << i;
-      }
-      edge = 4 * j + (q == 0 ? (mask ? __ffs(mask) - 1 : 0) : (mask ? 32 - __clz(mask) : 4));
-      if (mask != 0 || j == jend) break;
-      j += jstep;
-    }
-    const int other = __shfl_xor_sync(0xffffffffu, edge, 1);
-    if (has && q == 0) {
-      const int lo = win ? edge * 8 : 0, hi = win ? min(other * 8, len) : 0;
-      mh = max(lo, min(mh, hi - 1));
+    const PlanEntry e = plan_tile(a, mine, t, q);
+    if (live && t0 + ti / kPlanQ < T && q == 0) {
       const size_t pi = (size_t)t * a.plan_stride + row;
-      a.plan[pi] = any ? alpha : -INFINITY;
-      plan_i[np + pi] = lo | ((hi - lo) << 16);
-      plan_i[2 * np + pi] = mh;
-      if (hi > lo) {
-        atomicMin(&s_lo[t / kWinWarps], lo);
-        atomicMax(&s_hi[t / kWinWarps], hi);
+      a.plan[pi] = e.alpha;
+      plan_i[np + pi] = e.lo | ((e.hi - e.lo) << 16);
+      plan_i[2 * np + pi] = e.mh;
+      if (e.hi > e.lo) {
+        atomicMin(&s_lo[t / kWinWarps], e.lo);
+        atomicMax(&s_hi[t / kWinWarps], e.hi);
       }
     }
   }
@@ -357,40 +178,139 @@ template void plan_pass<1>(cudaStream_t, BandTable<1>&);
 template void plan_pass<2>(cudaStream_t, BandTable<2>&);
 template void plan_pass<kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&);
 
+namespace {
+
+// Longest rows (inputs and outputs) of a one-kernel product, and its tiles per CTA.  us per pass, two kernels
+// against one: 64^2 FP32 eps 60 4.9 / 3.2, 100^2 mixed eps 20 5.5 / 4.0, 256^2 mixed eps 64 6.1 / 4.2, eps
+// 13 13.8 / 11.6, 257^2 FP32 eps 130 9.5 / 8.5, 512^2 mixed eps 64 9.9 / 7.8, eps 13 17.5 / 15.1; at
+// 1024^2, where staging every row for each part costs more than the launch, 25.5 / 31.2 (eps 52) and
+// 21.4 / 21.3 (eps 209).  16 tiles per CTA took 5.2 us at 256^2 and 8.3 at 512^2 (eps 130; 7.1 with 8), 4
+// tiles 4.0 and 7.5.
+constexpr int kSmallLen = 512;
+constexpr int kSmallTiles = 8;
+
+// Make a table that of a one-kernel pass: CTAs of `group` rows, a warp per tile (exact sums: up to 16 warps,
+// the row's tiles among them).
+template <int MAXP>
+void small_table(BandTable<MAXP>& t) {
+  int chunks = 1;
+  finish(t, &chunks);
+  const int group = t.p[0].group;
+  int ctas = 0, tiles = 1, pitch = 16;
+  for (int q = 0; q < t.n; ++q) {
+    BandArgs& a = t.p[q];
+    int share = a.n_tiles;
+    a.parts = 1;
+    if (group == 8) {
+      a.parts = (a.n_tiles + kSmallTiles - 1) / kSmallTiles;
+      share = (a.n_tiles + a.parts - 1) / a.parts;
+      a.parts = (a.n_tiles + share - 1) / share;          // (no empty part)
+    }
+    a.plan_base = ctas;
+    ctas += (a.n_rows + group - 1) / group * a.parts;
+    tiles = std::max(tiles, share);
+    pitch = std::max(pitch, stage_pitch(t.p[q].len));
+  }
+  int warps = 4;
+  while (warps < tiles && warps < kSmallWarps) warps *= 2;
+  t.plans = ctas;
+  t.plan_items = tiles;
+  t.pitch_max = pitch;
+  t.plan_tpr_log2 = 0;
+  while ((group << t.plan_tpr_log2) < 32 * warps) ++t.plan_tpr_log2;
+}
+
 template <int MODE, int MAXP>
-void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
+void exact_pass(cudaStream_t s, BandTable<MAXP>& t) {
+  small_table(t);
+  ktimer_begin(s, kKPlan);
+  small_exact_launch<MODE, MAXP>(s, t);
+  ktimer_end(s);
+}
+
+}  // namespace
+
+template <int MODE, int MAXP>
+int band_pass(cudaStream_t s, BandTable<MAXP>& t, int form) {
+  bool exact = true, small = MAXP <= 2;
+  for (int q = 0; q < t.n; ++q) {
+    exact = exact && t.p[q].group == 2;
+    small = small && t.p[q].group == 8 && std::max(t.p[q].len, t.p[q].n_out) <= kSmallLen;
+  }
+  // Exact sums: one kernel at every size (us per pass against plan and sums apart: 64^2 3.4 / 5.7, 256^2
+  // 6.4 / 11.1, 512^2 13.7 / 21.8, 1024^2 37 / 56, 2048^2 132 / 204, all at eps 1).  A batch's pass is
+  // two launches whatever its eps: half of the problems each.
+  if (exact) {
+    if (MAXP <= 2 || t.n == 1) {
+      exact_pass<MODE>(s, t);
+      return 1;
+    }
+    size_t all = 0, head = 0;
+    for (int q = 0; q < t.n; ++q) all += (size_t)t.p[q].n_rows * t.p[q].n_out;
+    int cut = 0;
+    while (cut < t.n - 1 && (cut == 0 || 2 * head < all)) head += (size_t)t.p[cut].n_rows * t.p[cut].n_out, ++cut;
+    BandTable<MAXP> rest = t;
+    rest.n = t.n - cut;
+    std::copy(t.p + cut, t.p + t.n, rest.p);
+    t.n = cut;
+    exact_pass<MODE>(s, t);
+    exact_pass<MODE>(s, rest);
+    t.n += rest.n;
+    return 2;
+  }
+  if constexpr (MAXP <= 2) {
+    if (small) {
+      small_table(t);
+      ktimer_begin(s, kKPlan);
+      if (form == kFormFp32)
+        small_launch<MODE, kFormFp32, MAXP>(s, t);
+      else if (form == kFormSplit)
+        small_launch<MODE, kFormSplit, MAXP>(s, t);
+      else
+        small_launch<MODE, kFormSingle, MAXP>(s, t);
+      ktimer_end(s);
+      return 1;
+    }
+  }
   plan_pass(s, t);
   ktimer_begin(s, form == kFormFp32 ? kKBand : kKTensor);
-  bool exact = true;
-  for (int q = 0; q < t.n; ++q) exact = exact && t.p[q].group == 2;
-  if (exact)
-    exact_launch<MODE, MAXP>(s, t);
-  else if (form == kFormFp32)
+  if (form == kFormFp32)
     window_launch<MODE, kFormFp32, MAXP>(s, t);
   else if (form == kFormSplit)
     window_launch<MODE, kFormSplit, MAXP>(s, t);
   else
     window_launch<MODE, kFormSingle, MAXP>(s, t);
   ktimer_end(s);
+  return 2;
 }
 
-template void band_pass<0, 1>(cudaStream_t, BandTable<1>&, int);
-template void band_pass<1, 1>(cudaStream_t, BandTable<1>&, int);
-template void band_pass<0, 2>(cudaStream_t, BandTable<2>&, int);
-template void band_pass<1, 2>(cudaStream_t, BandTable<2>&, int);
-template void band_pass<0, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
-template void band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
+template int band_pass<0, 1>(cudaStream_t, BandTable<1>&, int);
+template int band_pass<1, 1>(cudaStream_t, BandTable<1>&, int);
+template int band_pass<0, 2>(cudaStream_t, BandTable<2>&, int);
+template int band_pass<1, 2>(cudaStream_t, BandTable<2>&, int);
+template int band_pass<0, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
+template int band_pass<1, kMaxBatch>(cudaStream_t, BandTable<kMaxBatch>&, int);
 
-// the plan kernel stages eight rows: more than the default 48 KB from rows of 1152 on
-cudaError_t plan_configure() {
-  const int lim = (int)(kPlanRows * plan_row_floats(4096 / kCW) * sizeof(float)) + 2 * 256 * (int)sizeof(int);
-  cudaError_t e = cudaFuncSetAttribute(band_plan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(band_plan_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(band_plan_kernel<kMaxBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+// Kernel attributes for rows of up to `longest`: more than the default 48 KB of dynamic shared memory, which
+// the plan kernel (eight rows) takes from rows of 1152 on, the exact one (two rows) from about 2350.
+// The one-kernel products stay below it.
+cudaError_t plan_configure(int longest) {
+  constexpr size_t kDefault = 48 * 1024;
+  constexpr int kMaxLen = 4096;
+  const int chunks = (longest + kCW - 1) / kCW;
+  cudaError_t e = cudaSuccess;
+  if (kPlanRows * plan_row_floats(chunks) * sizeof(float) + 2 * 256 * sizeof(int) > kDefault) {
+    const int lim = (int)(kPlanRows * plan_row_floats(kMaxLen / kCW) * sizeof(float)) + 2 * 256 * (int)sizeof(int);
+    e = cudaFuncSetAttribute(band_plan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(band_plan_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(band_plan_kernel<kMaxBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  }
+  if (e == cudaSuccess && small_smem(2, stage_pitch(longest), plan_row_floats(chunks), (longest + 15) / 16) > kDefault)
+    e = small_exact_configure((int)small_smem(2, stage_pitch(kMaxLen), plan_row_floats(kMaxLen / kCW), (kMaxLen + 15) / 16));
   return e;
 }
+static_assert((16 + 8 * ((kSmallLen + 15) / 32 * 32 + 16 + 2 * (kSmallLen / 32 + 3) + kSmallLen / 32 * 40) +
+               3 * 8 * kSmallTiles) * sizeof(float) <= 48 * 1024, "one-kernel products");
 
 int default_wait_limit() { return kSpinDefault; }
 
@@ -465,20 +385,20 @@ void half_step_band(fot_ctx* c, const float* pot_in, const float* lmarg, double 
   BandTable<1> t{};
   t.n = 1;
   t.spin_limit = c->spin;
-  int64_t k = 2 * 2;
+  int64_t k = 0;
   // pass over the contiguous axis: rows of pot_in, outputs along cols, written [k][L]
   t.p[0] = band_args(c, pot_in, c->rows, c->cols, eps, (float)(1.4426950408889634 / eps));
   t.p[0].y = c->R;
   const uint4* tilt = tilt_for(c, eps, t.p[0].group == 8 ? t.p[0].tile_w : 0, &k);
   t.p[0].tilt = tilt;
-  band_pass<0>(c->stream, t, form);
+  k += band_pass<0>(c->stream, t, form);
   // pass over the row axis (input R[k][L], log2 units) with the fused potential update
   t.p[0] = band_args(c, c->R, c->cols, c->rows, eps, 1.f);
   t.p[0].tilt = tilt;
   t.p[0].y = pot_out;
   t.p[0].lmarg = lmarg;
   t.p[0].logsum = logsum;
-  band_pass<1>(c->stream, t, form);
+  k += band_pass<1>(c->stream, t, form);
   c->launches += k;
 }
 
@@ -489,7 +409,7 @@ void half_step_band_pair(fot_ctx* c, const float* inA, const float* inB, const f
   BandTable<2> t{};
   t.n = 2;
   t.spin_limit = c->spin;
-  int64_t k = 2 * 2;
+  int64_t k = 0;
   const uint4* tilt = nullptr;
   for (int pass = 0; pass < 2; ++pass) {
     for (int q = 0; q < 2; ++q) {
@@ -510,10 +430,7 @@ void half_step_band_pair(fot_ctx* c, const float* inA, const float* inB, const f
         a.logsum = q == 0 ? logsumA : logsumB;
       }
     }
-    if (pass == 0)
-      band_pass<0>(c->stream, t, form);
-    else
-      band_pass<1>(c->stream, t, form);
+    k += pass == 0 ? band_pass<0>(c->stream, t, form) : band_pass<1>(c->stream, t, form);
   }
   c->launches += k;
 }

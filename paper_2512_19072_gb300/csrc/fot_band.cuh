@@ -39,6 +39,7 @@ struct BandArgs {
   int tile_w;          // outputs per plan tile and window unit: 8, 16 or 32
   int group;           // rows per window unit: 8, or 2 where every unit takes exact window sums
   int n_chunks, n_tiles, plan_stride;
+  int parts;                   // one-kernel products: CTAs that share a row group's tiles
   int plan_base, item_base;    // first plan CTA and first window item of this problem
   int items_row, n_items;      // window items along the outputs of a row group, and in all
   int wide_span;               // items whose windows span more go first
@@ -97,9 +98,10 @@ void band_set_eps(BandArgs& a, double eps);
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale);
 
 // one pass of every problem of the table: the window plan, then the window sums (MODE 0:
-// log-sum output; MODE 1: potential update).  Two kernel launches.
+// log-sum output; MODE 1: potential update).  Returns the kernels launched: two, or one for small
+// problems.
 template <int MODE, int MAXP>
-void band_pass(cudaStream_t s, BandTable<MAXP>& t, int form);
+int band_pass(cudaStream_t s, BandTable<MAXP>& t, int form);
 
 // the window plan alone, for a table whose window kernel the caller launches (fot_moments.cu)
 template <int MAXP>

@@ -81,10 +81,9 @@ static void capture_solve(fot_batch* b, cudaStream_t st, const float* const* g, 
         a2.logsum = (half == 0 && it == iters - 1) ? c->S_last : nullptr;
         a2.tilt = a1.tilt;
       }
-      band_pass<0>(st, *tab, form);
+      k += band_pass<0>(st, *tab, form);
       std::copy(p2.begin(), p2.end(), tab->p);
-      band_pass<1>(st, *tab, form);
-      k += 4;
+      k += band_pass<1>(st, *tab, form);
     }
   }
   delete tab;

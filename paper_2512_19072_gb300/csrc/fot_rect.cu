@@ -22,7 +22,7 @@
 namespace fot {
 
 int default_wait_limit();
-cudaError_t plan_configure();
+cudaError_t plan_configure(int longest);
 
 namespace {
 
@@ -175,7 +175,7 @@ fot_status solve_rect(const T* g, int rows_in, int cols_in, const T* G, int rows
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const size_t ni = (size_t)rows_in * cols_in, no = (size_t)rows_out * cols_out;
   const size_t nr = std::max((size_t)cols_in * rows_out, (size_t)cols_out * rows_in);
-  if (kBanded && plan_configure() != cudaSuccess) {       // (no context need exist on this device)
+  if (kBanded && plan_configure(std::max(std::max(rows_in, cols_in), std::max(rows_out, cols_out))) != cudaSuccess) {   // (no context need exist on this device)
     cudaGetLastError();
     return FOT_ECUDA;
   }

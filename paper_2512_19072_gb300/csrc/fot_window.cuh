@@ -52,9 +52,9 @@
 //
 // Narrow tiles.  The range shrinks with the tile: where eps is too small for 16 outputs, tiles of 8
 // take the same product with the unused rows of T zero, always with FP32 operands.  Below that
-// (eps < 5) every output is summed exactly, one exponential per term, relative to e(mh, o), by a
-// kernel of its own (exact_pass_kernel): its windows are a few blocks long, and tiles of 4 with the
-// product were slower (256^2, eps 1: 16.6 against 11.5 us per pass; 64^2: 10.7 against 6.2).
+// (eps < 5) every output is summed exactly, one exponential per term, relative to e(mh, o), plan and
+// sums in one kernel (fot_small.cuh): the windows are a few blocks long, and tiles of 4 with the product
+// were slower (256^2, eps 1: 16.6 against 11.5 us per pass with two kernels; 64^2: 10.7 against 6.2).
 //
 // Segments.  A unit outside the bound (a window that spans the gap between two parts of a target,
 // mostly) is summed with FP32 operands in segments of its window short enough to be in range by
@@ -722,14 +722,41 @@ struct Unit {
   bool pairs, skip;
 };
 
+// The sums of a unit, once its rows are staged: 2 rows x 16 exact outputs, or a product of 8 rows
+// (tilt is loaded for tiles of 16 and 32).
+template <int MODE>
+__device__ __forceinline__ void exact_unit(const BandArgs& a, const Unit& u, unsigned long long* terms) {
+  const int lane = threadIdx.x & 31;
+  const RowView& rv = u.rv;
+  if ((lane & 15) == 0 && rv.wl > 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
+  exact_output<MODE>(a, u.row, u.k0 + (lane & 15), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
+}
+template <int MODE, int FORM>
+__device__ __forceinline__ void product_unit(const BandArgs& a, const Unit& u, const Tilt<FORM>& tilt, unsigned long long* terms) {
+  const int lane = threadIdx.x & 31;
+  const RowView& rv = u.rv;
+  const int W = __reduce_max_sync(0xffffffffu, rv.wl);
+  const int walk = unit_walk(0.5f * (float)a.tile_w, rv, W, a.c);
+  if (walk != 2 && lane == 0 && W > 0)
+    atomicAdd(terms + (FORM == kFormFp32 || a.tile_w < 16 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
+  const bool plain = walk == 0 && a.tile_w >= 16 && (rv.staged || W == 0) && !long_window(W, a.c);
+  if (plain) {
+    const float kc = (float)(u.k0 + (a.tile_w >> 1)) + a.shift;
+    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip)
+                       : gemm_unit<MODE, FORM, 16, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip))
+      return;
+  }
+  other_unit<MODE, FORM>(a, u.r0, u.k0, rv, W, plain ? 2 : walk, u.skip, terms);
+}
+
 // The start of a window CTA: read the item and this warp's plan entries, stage the rows; `meanwhile`
 // runs while they are on their way.  s_x: four -inf (padded to 64 bytes), then the rows.  False: the
 // warp has nothing to do.
 template <int MAXP, typename F>
-__device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const BandArgs& a, float* s_x, uint64_t* s_bar, Unit& u,
-                                          F meanwhile) {
+__device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const BandArgs& a, float* s_x, uint64_t* s_bar, bool pairs,
+                                          Unit& u, F meanwhile) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  u.pairs = a.group == 2;
+  u.pairs = pairs;
   if (tid == 0) {
     mbar_init(smem_addr(s_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -805,54 +832,23 @@ __device__ __forceinline__ bool open_unit(const BandTable<MAXP>& tab, const Band
   return __all_sync(0xffffffffu, ok) && tile < a.n_tiles;
 }
 
-// A pass whose problems all take exact sums: 2 rows x 16 outputs per warp.  Its own kernel for its
-// registers (12 CTAs per SM; inside the window kernel, with 4 or 5, a pass at 512^2 and eps 2 took
-// 25 us).
-template <int MODE, int MAXP>
-__global__ void __launch_bounds__(kWinThreads, 12) exact_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
-  extern __shared__ __align__(128) float s_x[];
-  __shared__ __align__(8) uint64_t s_bar;
-  const int lane = threadIdx.x & 31;
-  const BandArgs& a = tab.p[find_prob<MAXP, 1>(tab, (int)blockIdx.x)];
-  Unit u;
-  if (!open_unit(tab, a, s_x, &s_bar, u, []() {})) return;
-  const RowView& rv = u.rv;
-  if ((lane & 15) == 0 && rv.wl > 0)
-    atomicAdd(a.terms + 4 * (blockIdx.x & (kTermSlots - 1)) + 1, (unsigned long long)rv.wl * 16);
-  exact_output<MODE>(a, u.row, u.k0 + (lane & 15), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
-}
-
 template <int MODE, int FORM, int MAXP>
 __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window_pass_kernel(const __grid_constant__ BandTable<MAXP> tab) {
   extern __shared__ __align__(128) float s_x[];
   __shared__ __align__(8) uint64_t s_bar;
-  const int lane = threadIdx.x & 31;
   const BandArgs& a = tab.p[find_prob<MAXP, 1>(tab, (int)blockIdx.x)];
   Unit u;
   Tilt<FORM> tilt;
-  if (!open_unit(tab, a, s_x, &s_bar, u, [&]() {
-        if (a.tile_w >= 16 && a.group != 2) tilt.load(a, a.tile_w, true);
+  const bool pairs = MAXP > 2 && a.group == 2;            // (a batch with problems of both kinds)
+  if (!open_unit(tab, a, s_x, &s_bar, pairs, u, [&]() {
+        if (a.tile_w >= 16 && !pairs) tilt.load(a, a.tile_w, true);
       }))
     return;
   unsigned long long* terms = a.terms + 4 * (blockIdx.x & (kTermSlots - 1));
-  const RowView& rv = u.rv;
-  if (u.pairs) {
-    if ((lane & 15) == 0 && rv.wl > 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
-    exact_output<MODE>(a, u.row, u.k0 + (lane & 15), rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
-    return;
-  }
-  const int W = __reduce_max_sync(0xffffffffu, rv.wl);
-  const int walk = unit_walk(0.5f * (float)a.tile_w, rv, W, a.c);
-  if (walk != 2 && lane == 0 && W > 0)
-    atomicAdd(terms + (FORM == kFormFp32 || a.tile_w < 16 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
-  const bool plain = walk == 0 && a.tile_w >= 16 && (rv.staged || W == 0) && !long_window(W, a.c);
-  if (plain) {
-    const float kc = (float)(u.k0 + (a.tile_w >> 1)) + a.shift;
-    if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip)
-                       : gemm_unit<MODE, FORM, 16, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip))
-      return;
-  }
-  other_unit<MODE, FORM>(a, u.r0, u.k0, rv, W, plain ? 2 : walk, u.skip, terms);
+  if (u.pairs)
+    exact_unit<MODE>(a, u, terms);
+  else
+    product_unit<MODE, FORM>(a, u, tilt, terms);
 }
 
 // launch with programmatic dependence on the kernel before it in the stream: its set-up (and
@@ -873,11 +869,17 @@ void launch_dependent(K kernel, dim3 grid, int threads, size_t smem, cudaStream_
 }
 
 // dynamic shared memory of the window kernel: four -inf, eight rows (within the default 48 KB)
-__host__ __device__ inline size_t window_smem(int pitch, int rows = 8) { return (size_t)(16 + rows * pitch) * sizeof(float); }
+__host__ __device__ inline size_t window_smem(int pitch) { return (size_t)(16 + 8 * pitch) * sizeof(float); }
 
 template <int MODE, int FORM, int MAXP>
 void window_launch(cudaStream_t s, const BandTable<MAXP>& t);
+
+// one-kernel passes (fot_small.cuh): products of one operand form, exact sums and their dynamic shared
+// memory limit
+template <int MODE, int FORM, int MAXP>
+void small_launch(cudaStream_t s, const BandTable<MAXP>& t);
 template <int MODE, int MAXP>
-void exact_launch(cudaStream_t s, const BandTable<MAXP>& t);
+void small_exact_launch(cudaStream_t s, const BandTable<MAXP>& t);
+cudaError_t small_exact_configure(int bytes);
 
 }  // namespace fot

@@ -1,6 +1,6 @@
-// The window kernels (fot_window.cuh) of one operand form, in a translation unit of its own so
-// that the forms compile in parallel.
-#include "fot_window.cuh"
+// The window kernels (fot_window.cuh) and one-kernel passes (fot_small.cuh) of one operand form, in
+// a translation unit of its own so that the forms compile in parallel.
+#include "fot_small.cuh"
 
 namespace fot {
 
@@ -15,5 +15,15 @@ template void window_launch<0, kFormFp32, 2>(cudaStream_t, const BandTable<2>&);
 template void window_launch<1, kFormFp32, 2>(cudaStream_t, const BandTable<2>&);
 template void window_launch<0, kFormFp32, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
 template void window_launch<1, kFormFp32, kMaxBatch>(cudaStream_t, const BandTable<kMaxBatch>&);
+
+template <int MODE, int FORM, int MAXP>
+void small_launch(cudaStream_t s, const BandTable<MAXP>& t) {
+  launch_small<MODE, FORM, 8>(s, t);
+}
+
+template void small_launch<0, kFormFp32, 1>(cudaStream_t, const BandTable<1>&);
+template void small_launch<1, kFormFp32, 1>(cudaStream_t, const BandTable<1>&);
+template void small_launch<0, kFormFp32, 2>(cudaStream_t, const BandTable<2>&);
+template void small_launch<1, kFormFp32, 2>(cudaStream_t, const BandTable<2>&);
 
 }  // namespace fot

@@ -45,6 +45,40 @@ def test_ragged_units(fot_lib, prec, shape, eps):
     _check(fot_lib, prec, psi, eps, 1)
 
 
+# passes of one kernel and of two: both sides of the longest row of a one-kernel product (512), row
+# groups whose tiles divide unevenly among CTAs, exact rows with more tiles than warps (16), and
+# two-kernel passes with ragged units
+@pytest.mark.parametrize("prec", ["fp32", "mixed"])
+@pytest.mark.parametrize("shape,eps", [((9, 512), 30.0), ((512, 9), 9.0), ((17, 511), 100.0), ((513, 12), 30.0),
+                                       ((7, 545), 400.0), ((530, 3), 9.0), ((3, 1025), 1.5), ((1, 260), 0.7),
+                                       ((2, 2050), 3.0)])
+def test_one_and_two_kernel_passes(fot_lib, prec, shape, eps):
+    psi = f32(inputs.random_potential(*shape, scale=0.1 * max(shape) ** 2 + 3 * eps, seed=12, zero_frac=0.15))
+    _check(fot_lib, prec, psi, eps, 4)
+
+
+# a batch whose passes are all exact, all products, or of both kinds gives what single solves give
+@pytest.mark.parametrize("prec", ["fp32", "mixed"])
+@pytest.mark.parametrize("shapes,eps", [([(40, 33)], [1.0]), ([(40, 33), (64, 64), (9, 130)], [1.0, 2.0, 1.5]),
+                                        ([(40, 33), (600, 30)], [40.0, 60.0]),
+                                        ([(40, 33), (64, 64), (600, 30)], [1.0, 40.0, 2.0])])
+def test_batches_of_exact_and_product_problems(fot_lib, prec, shapes, eps):
+    B = fot_lib
+    P = {"fp32": B.FOT_FP32, "mixed": B.FOT_MIXED}[prec]
+    rng = np.random.default_rng(13)
+    gs = [to_dev(f32(rng.uniform(0.05, 1.0, size=s))) for s in shapes]
+    Gs = [to_dev(f32(rng.uniform(0.05, 1.0, size=s))) for s in shapes]
+    batch = B.fot_batch_create(shapes, P)
+    B.fot_batch_solve(batch, gs, Gs, np.repeat(np.asarray(eps)[:, None], 4, axis=1), 4)
+    for q, s in enumerate(shapes):
+        ctx = B.fot_create(*s, P)
+        B.fot_solve(ctx, gs[q], Gs[q], [eps[q]], 4)
+        for a, b in zip(B.fot_potentials(B.fot_batch_context(batch, q)), B.fot_potentials(ctx)):
+            assert np.array_equal(to_np(a), to_np(b)), q       # the same arithmetic
+        ctx.close()
+    batch.close()
+
+
 # windows over whole rows of 1500 and 1499: more than an item's staging buffer holds
 @pytest.mark.parametrize("prec", ["fp32", "mixed"])
 @pytest.mark.parametrize("shape", [(10, 1500), (10, 1499)])
