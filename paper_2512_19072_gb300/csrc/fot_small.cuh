@@ -55,12 +55,8 @@ __global__ void __launch_bounds__(RR == 8 ? 256 : 32 * kSmallWarps, 2) small_pas
   }
   const bool skip = error_latched(a.err);                 // an error is latched: write nothing
   if (!bulk) {
-    // rows that are not 16-byte aligned: plain loads, -inf up to the next multiple of 4
-    const int n4 = (a.len + 3) & ~3;
-    const float* src = a.x + (size_t)r0 * a.len;
-    for (int r = 0; r < nr; ++r)
-      for (int i = tid; i < n4; i += blockDim.x)
-        rows[r * pitch + i] = i < a.len ? __ldg(src + (size_t)r * a.len + i) : -INFINITY;
+    stage_unaligned(rows, pitch, a.x + (size_t)r0 * a.len, a.len, a.len, nr, tid, (int)blockDim.x);
+    async_loads_done();
   }
   __syncthreads();                                        // (the barrier's initialisation, the -inf, plain rows)
   const bool ok = !bulk || stage_wait(smem_addr(&s_bar), 0, tab.spin_limit, a.err);
