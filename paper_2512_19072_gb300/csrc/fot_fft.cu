@@ -172,8 +172,15 @@ __global__ void __launch_bounds__(256) intensity_loss_kernel(float* __restrict__
                                                              const double* __restrict__ parts, int n_parts, size_t N,
                                                              double* __restrict__ out) {
   __shared__ double s[256];
-  const double inv = 1.0 / cta_sum(parts, n_parts, s);
-  const float ih = (float)inv, il = (float)(inv - (double)ih);
+  __shared__ float s_inv[2];
+  const double total = cta_sum(parts, n_parts, s);
+  if (threadIdx.x == 0) {                                 // (FP64 division: once per CTA)
+    const double inv = 1.0 / total;
+    s_inv[0] = (float)inv;
+    s_inv[1] = (float)(inv - (double)s_inv[0]);
+  }
+  __syncthreads();
+  const float ih = s_inv[0], il = s_inv[1];
   float ah = 0.f, al = 0.f;                               // this thread's sum as a pair
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
     const float x = v[i], l = lb[i];

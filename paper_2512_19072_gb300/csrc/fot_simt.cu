@@ -272,8 +272,11 @@ __global__ void log_marginals_kernel(const float* __restrict__ g, const float* _
                                      float* __restrict__ la, float* __restrict__ lb,
                                      float* __restrict__ psi0, float psi0_val, int* err) {
   if (error_latched(err)) return;
-  const float lga = (float)log(tot[0]);
-  const float lgb = (float)log(tot[1]);
+  // (one FP64 logarithm per image and CTA: one per thread made this 35 us at 1024^2)
+  __shared__ float s_log[2];
+  if (threadIdx.x < 2) s_log[threadIdx.x] = (float)log(tot[threadIdx.x]);
+  __syncthreads();
+  const float lga = s_log[0], lgb = s_log[1];
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N;
        i += (size_t)gridDim.x * blockDim.x) {
     const float x = g[i], y = G[i];
