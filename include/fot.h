@@ -67,11 +67,10 @@ typedef enum {
                             own exact maximum (one exponential per term): the plain form */
   FOT_AUTO = 3,          /* batches only: time FOT_FP32 and FOT_MIXED on the batch when its
                             graph is built and keep the faster */
-  FOT_BF16 = 4           /* the banded product of FOT_MIXED with single BF16 operands: one product
-                            per term instead of three, up to 2^-7 relative error each (both
-                            operands rounded to 8 significant bits), so a half-step moves f or psi
-                            by at most 2^-6 eps (against 2^-15 eps for FOT_MIXED); single contexts
-                            only */
+  FOT_BF16 = 4           /* the banded product of FOT_MIXED with the row's operand in a single BF16
+                            (8 significant bits) and the tilt matrix split: two products per term
+                            instead of three; a half-step moves f or psi by at most 2^-6 eps (against
+                            2^-15 eps for FOT_MIXED); single contexts only */
 } fot_precision;
 
 typedef enum { FOT_EPS_PX2 = 0, FOT_EPS_PAPER = 1 } fot_eps_units;

@@ -8,7 +8,7 @@
 namespace fot {
 
 // Arithmetic of the window sums: FP32 operands (three TF32 products per term), split BF16
-// (three products), single BF16 (one).
+// (three products), single BF16 for the rows (two).
 enum WindowForm : int { kFormFp32 = 0, kFormSplit = 1, kFormSingle = 2 };
 
 // One problem's pass over rows of x: y[o][r] = log2 sum_m 2^(x[r][m] x_scale - (o + shift - m)^2 c).

@@ -38,7 +38,9 @@
 // steps at 1024^2 where the mean is 13).
 //
 // Operands.  kFormSplit: BF16 hi + lo parts, hi*hi + hi*lo + lo*hi (2^-16 relative per product);
-// kFormSingle: hi*hi; kFormFp32: TF32 hi + lo parts (2^-21), two m16n8k8 per step and product.
+// kFormSingle: X in one part, T in both (T is the same in every step of a window, so that its rounding would not
+// average out as X's does: with hi*hi alone an update was 1.5 times as far from 64 bits as with the operands of
+// a longer table); kFormFp32: TF32 hi + lo parts (2^-21), two m16n8k8 per step and product.
 //
 // Range.  With kmax = TN/2 and D the farthest window position from mh: a term that matters to
 // output kap has X >= 2^-(2 kmax D c) (alpha is e(mh, kc); the largest term at kap is at least
@@ -68,7 +70,8 @@
 // 200 iterations at 1024^2 (800 passes, plan and launch gaps included) went from 31.9 to 14.5 ms with
 // split BF16 and from 45.7 to 16.5 ms with FP32 operands (FFMA with the operands through shared memory
 // before); 100 iterations at 2048^2, split BF16, from 39.8 to 21.2 ms; 256^2 annealed from eps 64 to 1
-// over 300 iterations from 41.7 to 11.7 ms; 64^2 at eps 1, 200 iterations, from 14.5 to 4.6 ms.
+// over 300 iterations from 41.7 to 11.7 ms (8.9 with the one-kernel passes of fot_small.cuh); 64^2 at eps 1, 200
+// iterations, from 14.5 to 4.6 ms (2.7).
 #pragma once
 
 #include "fot_band.cuh"
@@ -455,7 +458,7 @@ __device__ __forceinline__ void window_product(const BandArgs& a, float kc, cons
     absorb();
     // the small products first, then hi * hi
 #pragma unroll
-    for (int part = FORM == kFormSingle ? 2 : 0; part < 3; ++part)
+    for (int part = 0; part < 3; part += FORM == kFormSingle ? 2 : 1)
 #pragma unroll
       for (int h = 0; h < NH; ++h)
 #pragma unroll
@@ -464,7 +467,7 @@ __device__ __forceinline__ void window_product(const BandArgs& a, float kc, cons
           for (int t = 0; t < MT; ++t) {
             const uint32_t* A = (part == 0 ? tilt.lo[t] : tilt.hi[t]) + 4 * h;
             const uint32_t* Bm = (part == 1 ? xl[v] : xh[v]) + (NH == 2 ? 2 * h : 0);
-            const bool first = part == (FORM == kFormSingle ? 2 : 0) && h == 0;
+            const bool first = part == 0 && h == 0;
             mma<FORM>(P[v][t], A, Bm[0], Bm[1], first);
           }
   }
