@@ -223,9 +223,10 @@ def _peaks():
 # ALU rooflines (per SM per clock, times 152 SMs and the maximum SM clock):
 #  - MUFU ex2: 32 lanes/clk/SM on sm_103 (GB300 doubles sm_100's special-function rate;
 #    ncu's sm__inst_executed_pipe_xu peak agrees), bound of the dense exact pass;
-#  - FP32 FFMA: 128 lanes/clk/SM = 256 flop/clk/SM, bound of the banded pass's GEMM loop.
+#  - mma.sync TF32: 512 multiply-adds/clk/SM (470-512 measured), three of which make one multiply-add
+#    of the FP32 form's window products.
 EX2_PER_CLK_PER_SM = 32
-FFMA_FLOP_PER_CLK_PER_SM = 256
+TF32_FLOP_PER_CLK_PER_SM = 1024
 N_SM = 152
 
 
@@ -235,9 +236,9 @@ N_SM = 152
 # capture must lose its entry (the bench line then reports traffic null).
 NCU_TRAFFIC = {
     ("tc_pass_kernel", 1024, "mixed"): {
-        "bytes": (4.548096e6 + 0.0 + 8.751104e6 + 5.376e3) / 2,
-        "source": "ncu --set full, one row-pass and one column-pass launch (mean), "
-                  "profiles/tc_pass_kernel_c3_1024_mixed.md"},
+        "bytes": (4.673536e6 + 0.0 + 8.868096e6 + 0.0) / 2,
+        "source": "ncu --set full, one row-pass and one column-pass launch (mean), the beam and targets of "
+                  "perf/cases.py at 1024^2, eps 209; profiles/banded_passes.md"},
 }
 
 
@@ -257,13 +258,13 @@ def _roofline(n, a, ktimes, work, loop_ms):
     t_ms, n_launch = ktimes[dom]
     sec = t_ms * 1e-3
     gemm, exact, tensor, dense = (w * steps for w in work)
-    dense -= 2.0 * n * n * n * steps            # the phase step's two moment passes (not in the loop)
+    dense = max(dense - 2.0 * n * n * n * steps, 0.0)   # the dense form's two moment passes (not in the loop)
     ex2_peak = EX2_PER_CLK_PER_SM * N_SM * clk_mhz * 1e6 / 1e12
-    ffma_peak = FFMA_FLOP_PER_CLK_PER_SM * N_SM * clk_mhz * 1e6 / 1e12
+    tf32_peak = TF32_FLOP_PER_CLK_PER_SM * N_SM * clk_mhz * 1e6 / 1e12
     if dom == "band_pass_kernel" and gemm >= exact:
-        roof = {"bound": "alu", "achieved": 2.0 * gemm / sec / 1e12, "peak": ffma_peak,
-                "unit": "TFLOP/s", "work": "2 flop (one FFMA) per window term of the tilted GEMM",
-                "peak_source": f"FP32 FFMA {FFMA_FLOP_PER_CLK_PER_SM} flop/clk/SM x {N_SM} SMs x "
+        roof = {"bound": "tensor", "achieved": 6.0 * gemm / sec / 1e12, "peak": tf32_peak,
+                "unit": "TFLOP/s", "work": "6 flop (three TF32 multiply-adds) per window term of the tilted product",
+                "peak_source": f"mma.sync TF32 {TF32_FLOP_PER_CLK_PER_SM} flop/clk/SM x {N_SM} SMs x "
                                f"{clk_mhz:.0f} MHz",
                 "exact_window_terms": exact / steps}
     elif dom == "band_pass_kernel":
@@ -274,8 +275,8 @@ def _roofline(n, a, ktimes, work, loop_ms):
     elif dom == "tc_pass_kernel":
         # algorithmic work of the dense separable iteration: 8 n^3 flop per iteration (2 n^3 per
         # axis pass: n rows x n outputs x n terms, one multiply-add each), over the time of the
-        # tensor kernel's own launches; the flops it executed (3 BF16 multiply-adds per window
-        # term of the union windows) are reported beside it
+        # window kernel's own launches; the flops it executed (3 BF16 multiply-adds per window
+        # term) are reported beside it
         peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0)))
         algo = 8.0 * n ** 3 * a.iters * steps
         roof = {"bound": "tensor", "achieved": algo / sec / 1e12, "peak": peak,
@@ -291,7 +292,7 @@ def _roofline(n, a, ktimes, work, loop_ms):
         roof = {"bound": "alu", "achieved": dense / sec / 1e12, "peak": ex2_peak, "unit": "Tex2/s",
                 "work": "one exponential per (row, output, term) of the dense pass",
                 "peak_source": f"MUFU ex2 {EX2_PER_CLK_PER_SM}/clk/SM x {N_SM} SMs x {clk_mhz:.0f} MHz"}
-    else:                                        # window plan: reads the row, writes the plan
+    else:                                        # window plan (or whole one-kernel passes): reads the rows
         nbytes = n_launch * (n * n * 4 + n * ((n + 15) // 16) * 12)
         peak = float(peaks.get("hbm_gbs", 6800.0))
         roof = {"bound": "hbm", "achieved": nbytes / sec / 1e9, "peak": peak, "unit": "GB/s",
