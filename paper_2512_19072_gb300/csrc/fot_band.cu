@@ -138,8 +138,12 @@ void band_set_eps(BandArgs& a, double eps) {
   a.tile_w = tw == 0 ? 16 : tw;
   a.group = tw == 0 ? 2 : 8;
   a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
-  if (tw != 0)
-    for (int i = 0; i <= 32; ++i) a.step[i] = (float)exp2(32.0 * (i - 16) * (double)a.c);
+  if (tw == 0) return;
+  for (int i = 0; i <= 32; ++i) {
+    const double e = 32.0 * (i - 16) * (double)a.c;
+    a.step[i] = (float)exp2(e);
+    a.step_err[i] = (float)((e - log2((double)a.step[i])) / 16.0);
+  }
 }
 
 BandArgs band_args(fot_ctx* c, const float* x, int n_rows, int len, double eps, float x_scale) {

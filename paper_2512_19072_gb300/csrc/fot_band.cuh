@@ -46,7 +46,8 @@ struct BandArgs {
   int vec;                     // bit 0: rows of x are 16-byte aligned; bit 1: pairs of outputs are
                                // 8-byte aligned
   float step[33];              // 2^(32 kap c), kap = i - 16: the accumulators' scale per window
-                               // step, rounded once from 64 bits (its error grows with the steps)
+                               // step, rounded once from 64 bits
+  float step_err[33];          // log2 of what that rounding leaves out, per position of the walk
 };
 
 constexpr int kMaxBatch = 64;

@@ -180,6 +180,14 @@ __device__ __forceinline__ bool moment_unit(const BandArgs& a, int r0, int k0, f
     }
   }
   if (__any_sync(0xffffffffu, bad)) return false;
+  if (W > kLongWalk) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float walk = (float)(__shfl_sync(0xffffffffu, rv.mh, 8 * q + 4 * u) - lo[u]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) rest[i][u] += step_rounding(a, (float)(8 * i - 8 + g), walk, false);
+    }
+  }
   if (skip) return true;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {

@@ -42,3 +42,32 @@ def test_products_of_fp32_operands_are_not_biased(fot_lib, shape, power):
     dense, _ = _logsum(B, B.FOT_FP32_DENSE, psi, eps)
     assert terms[0] > 0 and terms[1] == 0                   # products alone
     assert abs((banded - dense).mean().item()) <= 2.0 ** -22
+
+
+def _exact_logsum(psi, eps):
+    """The same in 64 bits, in the units the kernels write (log2 times ln 2 as FP32 has it)."""
+    def axis(x):
+        i = torch.arange(x.shape[1], dtype=torch.float64, device=x.device)
+        top = x.max(dim=1, keepdim=True).values
+        return (torch.log(torch.exp(x - top) @ torch.exp(-(i[:, None] - i) ** 2 / (2 * eps))) + top).T
+    ln2 = math.log(2)
+    return axis(axis(psi.double() / eps)) * (torch.tensor(ln2, dtype=torch.float32).item() / ln2)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "mixed"])
+@pytest.mark.parametrize("shape", [(1200, 900), (512, 508)])
+def test_long_windows_keep_their_precision(fot_lib, shape, precision):
+    """Windows of 70 steps (eps 5909; across the whole row at 512): the step scale's rounding, 2^-25, must
+    not be carried through the walk (35 steps to the largest term: 1e-6).  Bound on the mean square where
+    the log-sum is small, natural logarithm: per pass an operand's rounding (FP32: ex2 and the
+    exponent, 2^-22; BF16 pairs: 2^-17 averaged over a step's 16 positions, 2^-19 at worst) and a rounding of
+    the log-sum between the passes (its size is log(2 pi eps) / 2 = 5: 2^-22); twice that for both passes."""
+    B = fot_lib
+    eps = LOG2E * 2.0 ** 12
+    psi = _level_potential(shape, eps, 4)
+    got, _ = _logsum(B, {"fp32": B.FOT_FP32, "mixed": B.FOT_MIXED}[precision], psi, eps)
+    ref = _exact_logsum(psi, eps)
+    near = ref.abs() < 0.3
+    rms = (got - ref)[near].pow(2).mean().sqrt().item()
+    assert near.sum() > 1000
+    assert rms <= (2 * 2.0 ** -22 + 2 * 2.0 ** -22 if precision == "fp32" else 2 * (2.0 ** -19 + 2.0 ** -22)), rms
