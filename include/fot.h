@@ -62,7 +62,9 @@ typedef enum {
                             relative, accumulated in FP32), for small eps an exact windowed
                             log-sum-exp */
   FOT_MIXED = 1,         /* the same with split-BF16 operands (three products, 2^-16 relative) and
-                            FP32 log-domain potentials */
+                            FP32 log-domain potentials.  A pass along a side that is not a multiple
+                            of 4 (or over rows that are not 16-byte aligned) keeps FP32 operands, as
+                            do eps below about 12 and windows that jump */
   FOT_FP32_DENSE = 2,    /* FP32 on the CUDA cores, every output scans every term with its
                             own exact maximum (one exponential per term): the plain form */
   FOT_AUTO = 3,          /* batches only: time FOT_FP32 and FOT_MIXED on the batch when its
