@@ -68,7 +68,8 @@ __device__ __forceinline__ void exact_moments(const BandArgs& a, int row, int k0
     }
   }
   (void)vec;
-  moment_output<MODE>(a, (size_t)o * a.n_rows + row, wl > 0 && off != -INFINITY, off, log2f(s0), lo, s1 / s0, s2 / s0);
+  const bool some = wl > 0 && (off != -INFINITY || isnan(s0));
+  moment_output<MODE>(a, (size_t)o * a.n_rows + row, some, off, log2f(s0), lo, s1 / s0, s2 / s0);
 }
 
 template <int MODE>

@@ -13,9 +13,15 @@
 //    at its nearest distance to the tile) lies below LB - kCut holds only terms below 2^-kCut
 //    of every output of the tile; the window is the hull of the remaining blocks (found per
 //    32-wide chunk first, then narrowed from both ends).
+// A row with a NaN or +inf in it is not to pass for one without: its blocks' maxima keep either (as
+// kWild), every one of its windows is the whole row and its offsets are NaN, so that the sums
+// come out as NaN (or are taken exactly, should the row hold values beyond kWild / 3).
+//
 // Arg-maxima carry the index in the low mantissa bits of the value they compare (5 bits for a
 // position, 7 for a chunk): one maximum instead of a compare and two selects; a chunk's maximum
-// is rounded by 2^-18 of itself that way, far inside the margin of kCut.
+// is rounded by up to 2^-16 of itself that way.  An offset that this takes from a lesser chunk (where the
+// values differ by less than that) only widens the window, and raises the operands: sums beyond
+// the range of FP32 are done again in segments or exactly.
 //
 // What bounds it: latency and issue slots (4 MB of input at 1024^2, in L2).  Two lanes serve a
 // (row, tile): each takes every other pair of chunks (packed FP32 pairs), half of the scanned
@@ -31,6 +37,7 @@ constexpr int kPlanRows = 8;                  // rows of a CTA: one row group of
 constexpr int kPlanThreads = 512;
 constexpr int kPlanQ = 2;                     // lanes per (row, tile)
 constexpr int kZS = kCW + 4;                  // words of a staged chunk
+constexpr float kWild = 3e38f;                // block maximum that stands for NaN and +inf
 
 // shared memory of one row (floats): chunk maxima and minus their positions (rounded up to four
 // chunks each), block maxima [n_chunks * 4], z [n_chunks * kZS]
@@ -43,6 +50,13 @@ __device__ __forceinline__ float tagged(float v, int index) {
 }
 template <int BITS>
 __device__ __forceinline__ int tag_of(float v) { return (int)(__float_as_uint(v) & ((1u << BITS) - 1u)); }
+
+// the larger of two values, NaN when either is
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
+}
 
 // Stage one row: blocks of 8 positions, a thread each (ti of tpr threads); four neighbouring threads
 // share a chunk.  load(m0, v): positions m0 .. m0 + 7, -inf outside the row.
@@ -62,9 +76,10 @@ __device__ __forceinline__ void plan_stage(const BandArgs& a, float* row_smem, i
 #pragma unroll
     for (int u = 0; u < 8; u += 2) {
       unpack2(mul2(pack2(v[u], v[u + 1]), sc2), v[u], v[u + 1]);
-      best = fmaxf(best, fmaxf(v[u], v[u + 1]));
+      best = max_nan(best, max_nan(v[u], v[u + 1]));
       top = fmaxf(top, fmaxf(tagged<5>(v[u], u0 + u), tagged<5>(v[u + 1], u0 + u + 1)));
     }
+    if (!(best <= kWild)) best = kWild;
     if (j < nch) {
       float4* const zb = reinterpret_cast<float4*>(z + j * kZS + u0);
       zb[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -116,6 +131,7 @@ __device__ __forceinline__ PlanEntry plan_tile(const BandArgs& a, const float* r
 #pragma unroll
   for (int d = 1; d < kPlanQ; d <<= 1) vb = fmaxf(vb, __shfl_xor_sync(0xffffffffu, vb, d));
   const bool any = vb != -INFINITY;                     // some term is finite
+  const bool wild = vb > kWild / 3.f;
   const int jb = any ? tag_of<7>(vb) : 0;
 
   // the maximum over that chunk (half of it for each lane)
@@ -203,10 +219,10 @@ __device__ __forceinline__ PlanEntry plan_tile(const BandArgs& a, const float* r
   }
   const int other = __shfl_xor_sync(0xffffffffu, edge, 1);
   PlanEntry e;
-  e.lo = win ? edge * 8 : 0;
-  e.hi = win ? min(other * 8, a.len) : 0;
+  e.lo = win && !wild ? edge * 8 : 0;
+  e.hi = wild ? a.len : win ? min(other * 8, a.len) : 0;
   e.mh = max(e.lo, min(mh, e.hi - 1));
-  e.alpha = any ? alpha : -INFINITY;
+  e.alpha = wild ? NAN : any ? alpha : -INFINITY;
   return e;
 }
 

@@ -688,7 +688,7 @@ __device__ __noinline__ bool segmented_unit(const BandArgs& a, int r0, int k0, c
   constexpr int NO = TN < 16 ? 1 : TN / 8;
   const float kc = (float)(k0 + TN / 2) + a.shift, c = a.c;
   const int L = min((int)(kRangeMax / (2.f * TN * c)) & ~15, 4096);   // TN (D + mh - lo) c <= TN 2 L c
-  if (L < 16) return false;
+  if (L < 16 || __any_sync(0xffffffffu, isnan(rv.alpha))) return false;   // (a row for exact sums: fot_plan.cuh)
   Tilt<kFormFp32> tilt;
   tilt.load(a, TN, false);
   float A[NO][2], T[NO][2];                               // the sums so far: offset and rest
