@@ -593,8 +593,9 @@ __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, flo
 
 // Exact window sum of one lane's output o of `row`, window [lo, lo + wl), xp[m] that row's position
 // m.  Terms are taken relative to e(mh, o), which is within the range of FP32 of the maximum unless
-// the maximum moves far from mh within the tile; a sum that overflows is done again from its exact
-// maximum.
+// the maximum moves far from mh within the tile, or exponents are so large (beyond 2^30) that their
+// rounding alone is; a sum out of range is done again from its exact maximum, and should that fail,
+// of terms rounded as the maximum is.
 template <int MODE>
 __device__ __forceinline__ void exact_output(const BandArgs& a, int row, int o, int lo, int wl, int mh, const float* xp,
                                              bool vec, bool skip) {
@@ -605,10 +606,12 @@ __device__ __forceinline__ void exact_output(const BandArgs& a, int row, int o, 
     float off = fmaf(dm * dm, nc, xp[mh] * sc);
     const f32x2 sc2 = pack2(sc, sc), nc2 = pack2(nc, nc), dn4 = pack2(-4.f, -4.f);
     const float d0 = fo - (float)lo;
+    float s0, s1;
+    auto in_range = [&]() { return s0 + s1 >= 1e-24f && s0 + s1 <= 3.4e38f; };   // (a NaN is not, and stays one)
     for (int pass = 0; pass < 2; ++pass) {
       const f32x2 no2 = pack2(-off, -off);
       f32x2 d01 = pack2(d0, d0 - 1.f);
-      float s0 = 0.f, s1 = 0.f;
+      s0 = s1 = 0.f;
 #pragma unroll 2
       for (int p = 0; p < wl; p += 4) {
         float e[4];
@@ -617,19 +620,24 @@ __device__ __forceinline__ void exact_output(const BandArgs& a, int row, int o, 
         s0 += ex2(e[0]) + ex2(e[1]);
         s1 += ex2(e[2]) + ex2(e[3]);
       }
-      const float sum = s0 + s1;
-      out = __fadd_rn(off, log2f(sum));
-      if (sum <= 3.4e38f) break;
-      // (a NaN ends here too and stays one)
-      off = -INFINITY;
+      if (in_range()) break;
+      // its exact maximum; then (the second time) terms rounded as that is
+      if (pass == 0) off = -INFINITY;
+      s0 = s1 = 0.f;
       d01 = pack2(d0, d0 - 1.f);
       for (int p = 0; p < wl; p += 4) {
         float e[4];
         exponents4(fetch4(xp, lo + p, wl - p, vec), sc2, pack2(0.f, 0.f), nc2, d01, e);
         d01 = add2(d01, dn4);
-        off = fmaxf(fmaxf(off, fmaxf(e[0], e[1])), fmaxf(e[2], e[3]));
+        if (pass == 0) {
+          off = fmaxf(fmaxf(off, fmaxf(e[0], e[1])), fmaxf(e[2], e[3]));
+        } else {
+          s0 += ex2(e[0] - off) + ex2(e[1] - off);
+          s1 += ex2(e[2] - off) + ex2(e[3] - off);
+        }
       }
     }
+    out = __fadd_rn(off, log2f(s0 + s1));
   }
   if (row >= a.n_rows || o >= a.n_out || skip) return;
   const size_t yi = (size_t)o * a.n_rows + row;
