@@ -39,7 +39,7 @@ __device__ __forceinline__ void moment_output(const BandArgs& a, size_t yi, bool
   }
 }
 
-// exact sums of 2 rows x 16 outputs (as exact_pair)
+// exact sums of 2 rows x 16 outputs
 template <int MODE>
 __device__ __forceinline__ void exact_moments(const BandArgs& a, int row, int k0, int lo, int wl, int mh, const float* xp,
                                               bool vec, bool skip) {
@@ -63,8 +63,10 @@ __device__ __forceinline__ void exact_moments(const BandArgs& a, int row, int k0
         s1 = fmaf(v, (float)p, s1);
         if (MODE == kMoment) s2 = fmaf(v, wr[lo + p], s2);
       }
-      if (s0 <= 3.4e38f && fabsf(s1) <= 3.4e38f) break;
-      off = top;                                          // out of range: again from the exact maximum
+      // out of range (s2 as well: its weights are as large as 1 / the pixel pitch): again from the exact
+      // maximum
+      if (s0 <= 3.4e38f && fabsf(s1) <= 3.4e38f && fabsf(s2) <= 3.4e38f) break;
+      off = top;
     }
   }
   (void)vec;
