@@ -280,6 +280,7 @@ extern "C" fot_status fot_backward(fot_ctx* c, const float* g, const float* G, c
   float *lxp = img(at_buf[8]), *lxn = img(at_buf[9]), *lyp = img(at_buf[10]), *lyn = img(at_buf[11]);
   float *pp = img(at_buf[12]), *pn = img(at_buf[13]), *R2 = img(at_buf[14]);
   const dim3 gN = grid_for(N);
+  tilt_begin(c);
   fill(c, neg_inf, N, -INFINITY);
   cudaMemsetAsync(mem + at_zero, 0, zero_bytes, s);
   // log(Lambda e^{in/eps} Lambda) of two inputs

@@ -366,6 +366,7 @@ static bool capture_loop(fot_ctx* c, const std::vector<double>& e) {
   if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
   c->stream = c->cap;
   loop_body(c, e);
+  tilt_reset(c);                           // (nothing has run)
   c->stream = user;
   cudaGraph_t g = nullptr;
   const bool ok = cudaStreamEndCapture(c->cap, &g) == cudaSuccess && g &&
@@ -664,6 +665,7 @@ fot_status fot_u_update(fot_ctx* c, const float* psi_in, double eps, float* f_ou
   if (!c || bad_ptr(psi_in) || bad_ptr(f_out) || !(eps > 0.0) || !isfinite(eps)) return FOT_EINVAL;
   if (!c->have_problem) return FOT_ESTATE;
   FOT_CUDA(cudaSetDevice(c->device));
+  tilt_begin(c);
   half_step(c, psi_in, c->la, eps, f_out, logsum_out);
   return check_launch(c);
 }
@@ -673,6 +675,7 @@ fot_status fot_v_update(fot_ctx* c, const float* f_in, double eps, float* psi_ou
   if (!c || bad_ptr(f_in) || bad_ptr(psi_out) || !(eps > 0.0) || !isfinite(eps)) return FOT_EINVAL;
   if (!c->have_problem) return FOT_ESTATE;
   FOT_CUDA(cudaSetDevice(c->device));
+  tilt_begin(c);
   half_step(c, f_in, c->lb, eps, psi_out, logsum_out);
   return check_launch(c);
 }

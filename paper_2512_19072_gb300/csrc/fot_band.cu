@@ -370,6 +370,14 @@ size_t tilt_bytes() { return (size_t)kTiltTables * kTiltWords * sizeof(uint4); }
 
 void tilt_reset(fot_ctx* c) { c->tilt_eps.clear(); }
 
+void tilt_begin(fot_ctx* c) {
+  if (!c->tilt) return;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+  c->captured = c->captured || st != cudaStreamCaptureStatusNone;
+  if (c->captured) tilt_reset(c);
+}
+
 void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
   if (!c->tilt) return;
   TiltArgs t{};

@@ -141,5 +141,9 @@ void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches);
 const uint4* tilt_for(fot_ctx* c, double eps, int tile_w, int64_t* launches);
 // forget what the device holds (the next use writes the tables again)
 void tilt_reset(fot_ctx* c);
+// At the start of an entry point whose passes run on the caller's stream: once a caller has captured such
+// a call, the table's writes are the caller's graphs' (now, or whenever one is replayed), so what the
+// host remembers of earlier calls no longer holds.
+void tilt_begin(fot_ctx* c);
 
 }  // namespace fot

@@ -107,6 +107,7 @@ static fot_status build_graph(fot_batch* b, const float* const* g, const float* 
   if (cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return FOT_ECUDA;
   int64_t k = 0;
   capture_solve(b, b->cap, g, G, eps, n_eps, iters, use_tc, &k);
+  for (fot_ctx* c : b->ctx) tilt_reset(c);   // (nothing has run)
   if (cudaStreamEndCapture(b->cap, &b->graph) != cudaSuccess) return FOT_ECUDA;
   if (cudaGraphInstantiate(&b->exec, b->graph, 0) != cudaSuccess) return FOT_ECUDA;
   b->nodes = k;
@@ -217,7 +218,6 @@ fot_status fot_batch_solve(fot_batch* b, const float* const* g, const float* con
     b->key_neps = n_eps;
   }
   if (cudaGraphLaunch(b->exec, b->stream) != cudaSuccess) return FOT_ECUDA;
-  for (fot_ctx* c : b->ctx) tilt_reset(c);   // (the tables hold what the graph last wrote)
   for (fot_ctx* c : b->ctx) {
     c->have_problem = true;
     c->have_solution = true;

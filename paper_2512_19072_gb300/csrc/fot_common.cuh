@@ -109,6 +109,7 @@ struct fot_ctx {
   // BF16 forms: tilt tables of the window sums (device) and the eps each was written for
   uint4* tilt = nullptr;
   std::vector<double> tilt_eps;
+  bool captured = false;     // a caller has captured half-steps of this context (tilt_begin)
   int spin = 0;              // polls of a bounded device wait
   int4* items = nullptr;     // item list of the window kernel
   int* order = nullptr;      // [2] its counters
