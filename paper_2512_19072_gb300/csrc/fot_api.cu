@@ -22,7 +22,7 @@ void set_problem_simt(fot_ctx* c, const float* g, const float* G, float* psi0, f
 void fill(fot_ctx* c, float* p, size_t N, float v);
 void source_stats(fot_ctx* c, const float* f, const float* S, double eps, double* out);
 bool intensity_supported(int rows, int cols);
-bool fft_tables(fot_ctx* c);
+fot_status fft_tables(fot_ctx* c);
 bool cfot_supported(int rows, int cols);
 void cfot_run(fot_ctx* c, const double* eps_px, int iters);
 size_t cfot_spectrum_floats();
@@ -455,7 +455,8 @@ fot_status fot_cfot_solve(fot_ctx* c, const float* g, const float* G, double dx,
     c->lam_hat = nullptr;
     return FOT_ENOMEM;
   }
-  if (!fft_tables(c)) return FOT_ENOMEM;
+  s = fft_tables(c);
+  if (s != FOT_OK) return s;
   s = start_solve(c, g, G, dx, eps, eps_units);
   if (s != FOT_OK) return s;
   std::vector<double> e((size_t)iters);
@@ -646,7 +647,7 @@ fot_status fot_intensity_loss(fot_ctx* c, const float* phi, double* loss_out, fl
   if (!c->have_problem) return FOT_ESTATE;
   if (!intensity_supported(c->rows, c->cols)) return FOT_EUNSUPPORTED;
   FOT_CUDA(cudaSetDevice(c->device));
-  if (!fft_tables(c)) return FOT_ENOMEM;
+  if (const fot_status t = fft_tables(c)) return t;
   double* out = c->red + 4 * c->red_blocks + 8;
   intensity_loss_gpu(c, phi, out);
   if (intensity_out)

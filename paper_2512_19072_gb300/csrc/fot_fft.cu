@@ -231,20 +231,31 @@ bool intensity_supported(int rows, int cols) {
 // one line of 4096, or eight of 512, stay within the default limit
 static_assert(fft_line_floats(kFftMax) * sizeof(float) + 8 * 16 <= 48 * 1024, "shared memory of a CTA's lines");
 
-bool fft_tables(fot_ctx* c) {
-  if (c->roots) return true;
+fot_status fft_tables(fot_ctx* c) {
+  if (c->roots) return FOT_OK;
+  if (!c->cap && cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    c->cap = nullptr;
+    return FOT_ECUDA;
+  }
   unsigned char* p = nullptr;
   constexpr size_t kRoots = kFftMax * sizeof(float2), kCos = kFftMax * sizeof(double);
   if (cudaMalloc((void**)&p, kRoots + kCos + 2 * kFftMax * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return FOT_ENOMEM;
+  }
+  // on the context's own stream, waited for: later calls may be on another stream, and the caller's may
+  // have work before it or be under capture
+  fft_roots_kernel<<<kFftMax / 256, 256, 0, c->cap>>>((float2*)p, (double*)(p + kRoots));
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->cap) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(p);
+    return FOT_ECUDA;
   }
   c->roots = (float2*)p;
   c->cosines = (double*)(p + kRoots);
   c->fft_parts = c->cosines + kFftMax;
-  fft_roots_kernel<<<kFftMax / 256, 256, 0, c->stream>>>(c->roots, c->cosines);
-  cudaStreamSynchronize(c->stream);                       // (once: later calls may be on another stream)
-  return true;
+  return FOT_OK;
 }
 
 // I / P into c->tmp and the loss into out[0] (device); c->R, c->R2 hold the spectrum between

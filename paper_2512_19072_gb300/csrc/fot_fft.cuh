@@ -198,7 +198,7 @@ inline int fft_lines_per_cta(int len, int n_lines) {
 }
 
 // the context's tables, made by its first transform: e^{-2 pi i k / 4096} in FP32 (c->roots), and
-// cos(2 pi k / 4096) in FP64 (c->cosines); false: no memory
-bool fft_tables(fot_ctx* c);
+// cos(2 pi k / 4096) in FP64 (c->cosines)
+fot_status fft_tables(fot_ctx* c);
 
 }  // namespace fot
