@@ -14,7 +14,7 @@
 // transforms those lines (the columns), writes |.|^2 at the shifted position and the CTA's part of
 // the total power.  A last pass divides by the total (every CTA adds the same parts in the same
 // order) and sums |I / P - b|; b = e^{log b} and the difference are formed in pairs of FP32 numbers
-// and summed that way per thread (2^-31 relative and better: a double exponential per pixel took
+// and summed that way per thread (2^-37 relative: a double exponential per pixel took
 // 33 us at 1024^2, the GPU's FP64 rate being 1/64 of its FP32 rate), across threads in FP64.
 #include "fot_fft.cuh"
 
@@ -46,7 +46,7 @@ __device__ __forceinline__ void small_dft(float (&re)[8], float (&im)[8], int le
   }
 }
 
-// (ah, al) += t, the rounding error of the sum kept in al
+// (ah, al) += t, the rounding error of the sum kept in al (Knuth's two-sum)
 __device__ __forceinline__ void pair_add(float& ah, float& al, float t) {
   const float sum = ah + t, z = sum - ah;
   al += (ah - (sum - z)) + (t - z);
@@ -134,24 +134,23 @@ __device__ double cta_sum(const double* __restrict__ v, int n, double* s) {
   return acc;
 }
 
-// e^l as hi + lo (relative error about 2^-31); l <= 0 or a little above
-__device__ __forceinline__ void exp_pair(float l, float& hi, float& lo) {
-  // l = n ln 2 + r: n times the leading 12 bits of ln 2 is exact, the rest as a small correction
-  const float n = rintf(l * kLog2e);
-  constexpr float kL1 = 0.693359375f;                     // 355 / 512
-  constexpr double kL2d = 0.69314718055994530942 - 0.693359375;
-  constexpr float kL2 = (float)kL2d, kL3 = (float)(kL2d - (double)kL2);
+// e^l as hi + lo, relative error below 2^-37; l <= 0 or a little above; tab: 2^(j/8) as hi + lo.  By table and
+// polynomial (Tang, "Table-driven implementation of the exponential function in IEEE floating-point
+// arithmetic", 1989): l = n ln(2) / 8 + r, e^l = 2^(n / 8) e^r, the product n ln(2) / 8 in three parts
+// of which the first is exact (Cody and Waite), |r| <= 0.044 as a pair.
+__device__ __forceinline__ void exp_pair(float l, const float2* tab, float& hi, float& lo) {
+  constexpr double kStep = 0.69314718055994530942 / 8.0;
+  const float n = rintf(l * (8.f * kLog2e));
+  constexpr float kL1 = 2839.f / 32768.f;                 // 12 bits of the step: n kL1 is exact
+  constexpr float kL2 = (float)(kStep - (double)kL1), kL3 = (float)(kStep - (double)kL1 - (double)kL2);
   const float r0 = fmaf(-n, kL1, l);                      // exact
   const float p = -n * kL2;
   const float pe = fmaf(-n, kL2, -p) - n * kL3;
-  const float rh = r0 + p, z = rh - r0;                   // r = rh + rl
+  const float rh = r0 + p, z = rh - r0;                   // r = rh + rl (Knuth's two-sum)
   const float rl = ((r0 - (rh - z)) + (p - z)) + pe;
-  // 1 + r + r^2 / 2 in pairs, r^3 (1/6 + r/24 + ...) in FP32
+  // 1 + r + r^2 / 2 in pairs (Dekker's fast two-sum), r^3 (1/6 + r/24 + ...), 2^-16 of the sum, in FP32
   const float q = rh * rh, qe = fmaf(rh, rh, -q) + 2.f * rh * rl;
-  float c = 1.f / 362880.f;
-  c = fmaf(c, rh, 1.f / 40320.f);
-  c = fmaf(c, rh, 1.f / 5040.f);
-  c = fmaf(c, rh, 1.f / 720.f);
+  float c = 1.f / 720.f;
   c = fmaf(c, rh, 1.f / 120.f);
   c = fmaf(c, rh, 1.f / 24.f);
   c = fmaf(c, rh, 1.f / 6.f);
@@ -159,12 +158,21 @@ __device__ __forceinline__ void exp_pair(float l, float& hi, float& lo) {
   const float h = 0.5f * q;
   const float s2 = s1 + h, e2 = h - (s2 - s1);
   const float tail = e1 + e2 + fmaf(c * rh, q, 0.5f * qe);
-  hi = s2 + tail;
-  lo = tail - (hi - s2);
-  const int k = (int)fminf(fmaxf(n, -300.f), 120.f);      // below 2^-126 the result fades to zero
+  const float eh = s2 + tail, el = tail - (eh - s2);
+  const int ni = (int)fminf(fmaxf(n, -2400.f), 960.f);    // below 2^-126 the result fades to zero
+  const float2 t = tab[ni & 7];
+  const float vh = eh * t.x, vl = fmaf(eh, t.x, -vh) + fmaf(eh, t.y, el * t.x);
+  const int k = ni >> 3;
   const float sa = exp2f((float)(k / 2)), sb = exp2f((float)(k - k / 2));
+  hi = vh + vl;
+  lo = (vl - (hi - vh)) * sa * sb;
   hi = hi * sa * sb;
-  lo = lo * sa * sb;
+}
+// 2^(j/8), j = 0 .. 7
+__device__ __forceinline__ double eighth_power(int j) {
+  return j == 0 ? 1.0 : j == 1 ? 1.0905077326652576592 : j == 2 ? 1.1892071150027210667 : j == 3 ? 1.2968395546510096659
+       : j == 4 ? 1.4142135623730950488 : j == 5 ? 1.5422108254079408236 : j == 6 ? 1.6817928305074290861
+                : 1.8340080864093424635;
 }
 
 // with P the total of the n_parts parts: v <- v / P in place and out[b] = sum |v / P - e^{lb}|
@@ -173,6 +181,12 @@ __global__ void __launch_bounds__(256) intensity_loss_kernel(float* __restrict__
                                                              double* __restrict__ out) {
   __shared__ double s[256];
   __shared__ float s_inv[2];
+  __shared__ float2 s_pow[8];
+  if (threadIdx.x < 8) {
+    const double v2 = eighth_power(threadIdx.x);
+    const float vh = (float)v2;
+    s_pow[threadIdx.x] = make_float2(vh, (float)(v2 - (double)vh));
+  }
   const double total = cta_sum(parts, n_parts, s);
   if (threadIdx.x == 0) {                                 // (FP64 division: once per CTA)
     const double inv = 1.0 / total;
@@ -187,10 +201,12 @@ __global__ void __launch_bounds__(256) intensity_loss_kernel(float* __restrict__
     const float qh = x * ih, ql = fmaf(x, ih, -qh) + x * il;
     v[i] = qh + ql;
     float bh = 0.f, bl = 0.f;
-    if (l != -INFINITY) exp_pair(l, bh, bl);
+    if (l != -INFINITY) exp_pair(l, s_pow, bh, bl);
     const float d = qh - bh, bb = qh - d, de = (bb - bh) + (qh - (d + bb));   // qh - bh = d + de
-    const float t = fabsf(d + (de + (ql - bl)));
-    pair_add(ah, al, t);
+    const float w = de + (ql - bl), th = d + w, tz = th - d;
+    const float tl = (d - (th - tz)) + (w - tz);          // |difference| = |th + tl|
+    pair_add(ah, al, fabsf(th));
+    al += th < 0.f ? -tl : tl;
   }
   s[threadIdx.x] = (double)ah + (double)al;
   __syncthreads();
