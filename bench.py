@@ -292,12 +292,30 @@ def _roofline(n, a, ktimes, work, loop_ms):
         roof = {"bound": "alu", "achieved": dense / sec / 1e12, "peak": ex2_peak, "unit": "Tex2/s",
                 "work": "one exponential per (row, output, term) of the dense pass",
                 "peak_source": f"MUFU ex2 {EX2_PER_CLK_PER_SM}/clk/SM x {N_SM} SMs x {clk_mhz:.0f} MHz"}
-    else:                                        # window plan (or whole one-kernel passes): reads the rows
-        nbytes = n_launch * (n * n * 4 + n * ((n + 15) // 16) * 12)
-        peak = float(peaks.get("hbm_gbs", 6800.0))
-        roof = {"bound": "hbm", "achieved": nbytes / sec / 1e9, "peak": peak, "unit": "GB/s",
-                "work": "x read once + 3 plan words per (row, tile) written",
-                "peak_source": "STREAM copy, " + peak_src}
+    else:
+        # window plans, and whole passes whose plan and sums are one kernel.  Where no pass had a window
+        # kernel, all the terms are theirs and no plan goes through memory; else the plans' bytes, and the
+        # exponentials of the exact passes among them.  The bound is what takes longest at its peak.
+        whole = ktimes["band_pass_kernel"][1] + ktimes["tc_pass_kernel"][1] == 0
+        hbm = float(peaks.get("hbm_gbs", 6800.0))
+        nbytes = n_launch * (2 * n * n * 4 if whole else n * n * 4 + n * ((n + 15) // 16) * 12)
+        parts = [{"bound": "hbm", "achieved": nbytes / sec / 1e9, "peak": hbm, "unit": "GB/s",
+                  "work": "input read once, output written once" if whole else
+                          "x read once + 3 plan words per (row, tile) written",
+                  "peak_source": "STREAM copy, " + peak_src},
+                 {"bound": "alu", "achieved": exact / sec / 1e12, "peak": ex2_peak, "unit": "Tex2/s",
+                  "work": "one exponential per exact-window term",
+                  "peak_source": f"MUFU ex2 {EX2_PER_CLK_PER_SM}/clk/SM x {N_SM} SMs x {clk_mhz:.0f} MHz"}]
+        if whole:
+            parts.append({"bound": "tensor", "achieved": 6.0 * gemm / sec / 1e12, "peak": tf32_peak, "unit": "TFLOP/s",
+                          "work": "6 flop (three TF32 multiply-adds) per window term of the tilted product",
+                          "peak_source": f"mma.sync TF32 {TF32_FLOP_PER_CLK_PER_SM} flop/clk/SM x {N_SM} SMs x "
+                                         f"{clk_mhz:.0f} MHz"})
+            parts.append({"bound": "tensor", "achieved": 6.0 * tensor / sec / 1e12,
+                          "peak": float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0))),
+                          "unit": "TFLOP/s", "work": "3 BF16 multiply-adds (split precision) per window term computed",
+                          "peak_source": "cuBLAS bf16 sustained, " + peak_src})
+        roof = max(parts, key=lambda p: p["achieved"] / p["peak"])
     tr = NCU_TRAFFIC.get((dom, n, a.precision))
     roof.update({"kernel": dom, "frac": roof["achieved"] / roof["peak"],
                  "traffic": tr["bytes"] if tr else None,
