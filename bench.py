@@ -230,10 +230,17 @@ TF32_FLOP_PER_CLK_PER_SM = 1024
 N_SM = 152
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a kernel, from an ncu
-# capture of the current build on the benchmark workload (the capture and its command are in the
-# named profiles/ summary).  Keyed by (kernel, n, precision); a kernel that changes since its
-# capture must lose its entry (the bench line then reports traffic null).
+# the kernels of each timing class (binding.KERNEL_CLASS_NAMES)
+CLASS_KERNELS = {"band_plan_kernel": "band_plan_kernel, small_pass_kernel",
+                 "band_pass_kernel": "window_pass_kernel, FP32 operands",
+                 "tc_pass_kernel": "window_pass_kernel, BF16 operands",
+                 "axis_pass_kernel": "axis_pass_kernel"}
+
+
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a kernel class, from an
+# ncu capture on the inputs that the source names (the capture and its command are in the named
+# profiles/ summary).  Keyed by (class, n, precision); a kernel that changes since its capture
+# must lose its entry (the bench line then reports traffic null).
 NCU_TRAFFIC = {
     ("tc_pass_kernel", 1024, "mixed"): {
         "bytes": (4.673536e6 + 0.0 + 8.868096e6 + 0.0) / 2,
@@ -317,7 +324,7 @@ def _roofline(n, a, ktimes, work, loop_ms):
                           "peak_source": "cuBLAS bf16 sustained, " + peak_src})
         roof = max(parts, key=lambda p: p["achieved"] / p["peak"])
     tr = NCU_TRAFFIC.get((dom, n, a.precision))
-    roof.update({"kernel": dom, "frac": roof["achieved"] / roof["peak"],
+    roof.update({"kernel": CLASS_KERNELS[dom], "frac": roof["achieved"] / roof["peak"],
                  "traffic": tr["bytes"] if tr else None,
                  "traffic_source": tr["source"] if tr else None,
                  "launches": n_launch, "avg_launch_us": t_ms * 1e3 / max(n_launch, 1),

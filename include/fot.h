@@ -159,8 +159,8 @@ fot_status fot_select_eps(fot_ctx* ctx, const float* g, const float* G, double d
  *   eps in px^2 (n_eps == 1, or n_eps == iters for one value per iteration); f_out
  *   (rows_in x cols_in) and psi_out (rows_out x cols_out): device buffers of the caller that
  *   receive the potentials (px^2, -inf at zero mass); cuda_stream: the stream (NULL: default).
- * The call allocates and frees its temporaries (3 images, a window plan of 3 words per 16 pixels
- * and a few words) and synchronises the
+ * The call allocates and frees its temporaries (3 images, a window plan of 3 words and an
+ * item list of half a byte per 8 pixels, and a few words) and synchronises the
  * stream before returning.  Errors: FOT_EINVAL (a null pointer, a size < 1 or > 3072,
  * iters < 1, n_eps other than 1 or iters, eps not finite and > 0), FOT_EMASS (g or G without
  * mass), FOT_ENOMEM, FOT_ENONFINITE (a non-finite potential), FOT_ECUDA. */
@@ -339,7 +339,7 @@ fot_status fot_loop_time(fot_ctx* ctx, double* ms_out, int64_t* passes_out);
  * evaluated since creation: rows*len*len per dense pass, the window sizes for banded passes
  * (each term is one multiply-add of the exp-domain contraction); tensor_terms_out (may be
  * NULL) receives the part computed from BF16 operands (each term there is three BF16
- * multiply-adds of the split-precision product).  Synchronising. */
+ * multiply-adds of the split-precision product, two with FOT_BF16).  Synchronising. */
 fot_status fot_work_count(fot_ctx* ctx, int64_t* terms_out, int64_t* tensor_terms_out);
 
 /* The same count split by how the terms were evaluated: out4[0] banded products of FP32

@@ -1,5 +1,5 @@
 // Banded axis pass: arguments and entry points shared by the plan and window kernels
-// (fot_band.cu, fot_window.cu), the single-problem half-step and the batched solver
+// (fot_band.cu, fot_window.cuh), the single-problem half-step and the batched solver
 // (fot_batch.cu).
 #pragma once
 

@@ -42,7 +42,7 @@ __device__ __forceinline__ void moment_output(const BandArgs& a, size_t yi, bool
 // exact sums of 2 rows x 16 outputs
 template <int MODE>
 __device__ __forceinline__ void exact_moments(const BandArgs& a, int row, int k0, int lo, int wl, int mh, const float* xp,
-                                              bool vec, bool skip) {
+                                              bool skip) {
   const int o = k0 + (threadIdx.x & 15);
   if (row >= a.n_rows || o >= a.n_out || skip) return;
   const float fo = (float)o + a.shift, sc = a.x_scale, c = a.c;
@@ -69,7 +69,6 @@ __device__ __forceinline__ void exact_moments(const BandArgs& a, int row, int k0
       off = top;
     }
   }
-  (void)vec;
   const bool some = wl > 0 && (off != -INFINITY || isnan(s0));
   moment_output<MODE>(a, (size_t)o * a.n_rows + row, some, off, log2f(s0), lo, s1 / s0, s2 / s0);
 }
@@ -82,7 +81,7 @@ __device__ __noinline__ void exact_moment_unit(const BandArgs& a, int r0, int k0
     const int l = __shfl_sync(0xffffffffu, rv.lo, src), w = __shfl_sync(0xffffffffu, rv.wl, src);
     const int m = __shfl_sync(0xffffffffu, rv.mh, src);
     const float* xr = (const float*)__shfl_sync(0xffffffffu, (unsigned long long)rv.row, src);
-    exact_moments<MODE>(a, r0 + 2 * p + half, k0, l, w, m, xr, rv.vec, skip);
+    exact_moments<MODE>(a, r0 + 2 * p + half, k0, l, w, m, xr, skip);
   }
 }
 
@@ -221,7 +220,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) moment_pass_kernel(const __gri
   const RowView& rv = u.rv;
   if (u.pairs) {
     if ((lane & 15) == 0 && rv.wl > 0) atomicAdd(terms + 1, (unsigned long long)rv.wl * 16);
-    exact_moments<MODE>(a, u.row, u.k0, rv.lo, rv.wl, rv.mh, rv.row, rv.vec, u.skip);
+    exact_moments<MODE>(a, u.row, u.k0, rv.lo, rv.wl, rv.mh, rv.row, u.skip);
     return;
   }
   const int W = __reduce_max_sync(0xffffffffu, rv.wl);

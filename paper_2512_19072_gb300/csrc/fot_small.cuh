@@ -96,7 +96,6 @@ __global__ void __launch_bounds__(RR == 8 ? 256 : 32 * kSmallWarps, 2) small_pas
   Unit u;
   u.r0 = r0;
   u.row = r0 + lr;
-  u.pairs = RR == 2;
   u.skip = skip;
   u.rv.staged = u.rv.vec = true;
   u.rv.row = rows + lr * pitch;
