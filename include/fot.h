@@ -160,7 +160,7 @@ fot_status fot_select_eps(fot_ctx* ctx, const float* g, const float* G, double d
  *   (rows_in x cols_in) and psi_out (rows_out x cols_out): device buffers of the caller that
  *   receive the potentials (px^2, -inf at zero mass); cuda_stream: the stream (NULL: default).
  * The call allocates and frees its temporaries (3 images, a window plan of 3 words and an
- * item list of half a byte per 8 pixels, and a few words) and synchronises the
+ * item list of half a byte per 16 pixels, and a few words) and synchronises the
  * stream before returning.  Errors: FOT_EINVAL (a null pointer, a size < 1 or > 3072,
  * iters < 1, n_eps other than 1 or iters, eps not finite and > 0), FOT_EMASS (g or G without
  * mass), FOT_ENOMEM, FOT_ENONFINITE (a non-finite potential), FOT_ECUDA. */

@@ -125,14 +125,17 @@ void finish(BandTable<MAXP>& t, int* max_chunks) {
 // the Gaussian has fallen by 2^-kCut, with mh in its middle: tile_w W c.  Real windows are longer
 // where the transport map jumps, so a width is taken while that estimate leaves room (the wider
 // tile shares each exponential, and each unit's set-up, between more outputs; units out of range
-// are summed in segments).  8 ends where exact sums become the faster ones (at 256^2, per pass:
-// eps 7 12.7 against 23.5 us, eps 5 13.0 against 10.3).
+// are summed in segments).  32 ends at eps 101 (us per pass, 32-wide against 16-wide: split BF16 at 1024^2,
+// eps 130 24.9 / 21.7, eps 80 31.2 / 22.8; FP32, eps 130 24.1 / 25.1, eps 80 26.1 / 25.1; 256^2, split BF16, eps 130
+// 4.75 / 4.21, eps 80 5.14 / 4.20: 32 is right for FP32 operands and costs the others up to 15 % between eps
+// 101 and 168).  16 ends at eps 12 (16-wide against exact, FP32: 1024^2 eps 11 37.7 / 32.7, eps 16 31.9 / 32.9, 2048^2 eps
+// 11 111 / 105, eps 13 100 / 105; below 1024^2 exact sums stay the faster ones to eps 20 and beyond: 512^2 eps 16
+// 14.3 / 10.7, 256^2 12.0 / 6.1).
 int tile_width_for(float c) {
   const float reach = 2.f * sqrtf(kCut / c);
   auto need = [&](float w) { return w * (w + reach) * c; };
   if (need(32.f) <= 42.f) return 32;
   if (need(16.f) <= 64.f) return 16;
-  if (need(8.f) <= 45.f) return 8;
   return 0;
 }
 
@@ -142,6 +145,7 @@ void band_set_eps(BandArgs& a, double eps) {
   const int tw = tile_width_for(a.c);
   a.tile_w = tw == 0 ? 16 : tw;
   a.group = tw == 0 ? 2 : 8;
+  // (1.8 and 3.6 for 2.6: within 1 % at 1024^2 and 2048^2, eps 209 and 839)
   a.wide_span = kWinWarps * a.tile_w + (int)(2.6f * sqrtf(kCut / a.c));
   if (tw == 0) return;
   for (int i = 0; i <= 32; ++i) {
@@ -193,8 +197,9 @@ namespace {
 // against one: 64^2 FP32 eps 60 4.9 / 3.2, 100^2 mixed eps 20 5.5 / 4.0, 256^2 mixed eps 64 6.1 / 4.2, eps
 // 13 13.8 / 11.6, 257^2 FP32 eps 130 9.5 / 8.5, 512^2 mixed eps 64 9.9 / 7.8, eps 13 17.5 / 15.1; at
 // 1024^2, where staging every row for each part costs more than the launch, 25.5 / 31.2 (eps 52) and
-// 21.4 / 21.3 (eps 209).  16 tiles per CTA took 5.2 us at 256^2 and 8.3 at 512^2 (eps 130; 7.1 with 8), 4
-// tiles 4.0 and 7.5.
+// 21.4 / 21.3 (eps 209).  Between them one kernel is still ahead at 640, the longest rows that could stay
+// within 48 KB (576^2 mixed eps 60 14.7 / 12.0, 640^2 mixed eps 130 14.0 / 10.7).  16 tiles per CTA took 5.2
+// us at 256^2 and 8.3 at 512^2 (eps 130; 7.1 with 8), 4 tiles 4.0 and 7.5.
 constexpr int kSmallLen = 512;
 constexpr int kSmallTiles = 8;
 
@@ -387,7 +392,7 @@ void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
     if (!c->tilt_eps.empty() && c->tilt_eps.back() == eps[i]) continue;
     const float cc = (float)(1.4426950408889634 / (2.0 * eps[i]));
     const int tw = tile_width_for(cc);
-    if (tw < 16) continue;                    // narrow tiles, exact windows: no table
+    if (tw == 0) continue;                    // exact windows: no table
     const int k = (int)c->tilt_eps.size();
     t.c[k] = cc;
     t.tw[k >> 2] |= tw << (8 * (k & 3));
@@ -401,7 +406,7 @@ void tilt_prepare(fot_ctx* c, const double* eps, int n, int64_t* launches) {
 }
 
 const uint4* tilt_for(fot_ctx* c, double eps, int tile_w, int64_t* launches) {
-  if (!c->tilt || tile_w < 16) return nullptr;
+  if (!c->tilt || tile_w == 0) return nullptr;
   for (size_t i = 0; i < c->tilt_eps.size(); ++i)
     if (c->tilt_eps[i] == eps) return c->tilt + i * kTiltWords;
   tilt_prepare(c, &eps, 1, launches);

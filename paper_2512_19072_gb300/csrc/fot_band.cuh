@@ -36,7 +36,7 @@ struct BandArgs {
   float coord0, coord_step;
   float x_scale, c, eps, shift;
   int n_rows, len, n_out;
-  int tile_w;          // outputs per plan tile and window unit: 8, 16 or 32
+  int tile_w;          // outputs per plan tile and window unit: 16 or 32
   int group;           // rows per window unit: 8, or 2 where every unit takes exact window sums
   int n_chunks, n_tiles, plan_stride;
   int parts;                   // one-kernel products: CTAs that share a row group's tiles
@@ -84,13 +84,13 @@ __device__ __forceinline__ int find_prob(const BandTable<MAXP>& t, int gi) {
   return lo;
 }
 
-// Tile width of a pass with kernel constant c: outputs per window unit, 32, 16 or 8; 0 where
+// Tile width of a pass with kernel constant c: outputs per window unit, 32 or 16; 0 where
 // eps is too small for the tilted product (the pass then runs exact window sums in units of 2 rows x 16
 // outputs).
 int tile_width_for(float c);
 
-// tiles of n outputs that a plan must have room for: 8-wide ones
-inline size_t plan_tiles(int n) { return ((size_t)n + 7) / 8; }
+// tiles of n outputs that a plan must have room for: 16-wide ones
+inline size_t plan_tiles(int n) { return ((size_t)n + 15) / 16; }
 
 // the fields of a pass that follow from eps: kernel constant, tile width, step scales
 void band_set_eps(BandArgs& a, double eps);

@@ -78,7 +78,7 @@ struct fot_ctx {
   float* tmp2 = nullptr;     // rows x cols scratch
   float* phi = nullptr;      // rows x cols phase (host-buffer entry point)
   float* col_phi = nullptr;  // rows: phase along the centre column
-  float* plan = nullptr;     // window plan of a banded pass: 3 words per (row, tile of 8 outputs or more)
+  float* plan = nullptr;     // window plan of a banded pass: 3 words per (row, tile of 16 outputs or more)
   double* red = nullptr;     // reduction scratch (partials + results)
   // tables of the transforms (one allocation, made by the first one) and their partial sums
   float2* roots = nullptr;

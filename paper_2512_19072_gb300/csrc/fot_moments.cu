@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) moment_pass_kernel(const __gri
   Unit u;
   Tilt<kFormFp32> tilt;
   if (!open_unit(tab, a, s_x, &s_bar, a.group == 2, u, [&]() {
-        if (a.group != 2) tilt.load(a, 16, false);
+        if (a.group != 2) tilt.load(a, 16);
       }))
     return;
   unsigned long long* terms = a.terms + 4 * (blockIdx.x & (kTermSlots - 1));

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(RR == 8 ? 256 : 32 * kSmallWarps, 2) small_pas
     }
   } else if (warp < T) {
     Tilt<FORM> tilt;
-    if (a.tile_w >= 16) tilt.load(a, a.tile_w, true);
+    tilt.load(a, a.tile_w);
     open(warp);
     product_unit<MODE, FORM>(a, u, tilt, terms);
   }

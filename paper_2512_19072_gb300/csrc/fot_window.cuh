@@ -52,11 +52,11 @@
 // gap).  An offset that lies too far below the maximum shows as an output that is not finite; such a
 // unit is summed again in segments.
 //
-// Narrow tiles.  The range shrinks with the tile: where eps is too small for 16 outputs, tiles of 8
-// take the same product with the unused rows of T zero, always with FP32 operands.  Below that
-// (eps < 5) every output is summed exactly, one exponential per term, relative to e(mh, o), plan and
-// sums in one kernel (fot_small.cuh): the windows are a few blocks long, and tiles of 4 with the product
-// were slower (256^2, eps 1: 16.6 against 11.5 us per pass with two kernels; 64^2: 10.7 against 6.2).
+// Small eps.  The range shrinks with the tile: where eps is too small for 16 outputs (below about 12) every
+// output is summed exactly, one exponential per term, relative to e(mh, o), plan and sums in one kernel
+// (fot_small.cuh): the windows are a few blocks long.  Products of 8-wide tiles, with half of T's rows
+// zero, were slower (us per pass, FP32, eps 7 / 11: 256^2 9.6 / 8.0 against 6.8 / 6.0 exact, 1024^2 46 / 44 against
+// 32 / 33) and twice as far from 64 bits (log-sums at eps 8: 2.5e-7 and 1.1e-7 rms).
 //
 // Segments.  A unit outside the bound (a window that spans the gap between two parts of a target,
 // mostly) is summed with FP32 operands in segments of its window short enough to be in range by
@@ -309,9 +309,8 @@ struct Tilt {
   static constexpr int NH = FORM == kFormFp32 ? 2 : 1;
   uint32_t hi[2][4 * NH], lo[2][4 * NH];
   f32x2 G[2][2];
-  // tw: outputs of the tile (16 and 8: first row tile only, 8: its second half zero); table:
-  // a.tilt holds the fragments (BF16 forms, tiles of 16 and 32)
-  __device__ __forceinline__ void load(const BandArgs& a, int tw, bool table) {
+  // tw: outputs of the tile (16: first row tile only); BF16 forms take a.tilt's fragments
+  __device__ __forceinline__ void load(const BandArgs& a, int tw) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
@@ -321,20 +320,15 @@ struct Tilt {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
           tilt_fragments_tf32(a.c, kap0, h, lane, hi[t] + 4 * h, lo[t] + 4 * h);
-          if (tw < 16) {
-            hi[t][4 * h + 1] = hi[t][4 * h + 3] = lo[t][4 * h + 1] = lo[t][4 * h + 3] = 0u;
-          }
         }
-      } else if (table) {
+      } else {
         const uint4 h4 = __ldg(a.tilt + t * 64 + lane), l4 = __ldg(a.tilt + t * 64 + 32 + lane);
         hi[t][0] = h4.x; hi[t][1] = h4.y; hi[t][2] = h4.z; hi[t][3] = h4.w;
         lo[t][0] = l4.x; lo[t][1] = l4.y; lo[t][2] = l4.z; lo[t][3] = l4.w;
-      } else {
-        tilt_fragments_bf16(a.c, kap0, lane, hi[t], lo[t]);
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float v = a.step[min(kap0 + (lane >> 2) + 8 * h, 15) + 16];
+        const float v = a.step[kap0 + (lane >> 2) + 8 * h + 16];
         G[t][h] = pack2(v, v);
       }
     }
@@ -344,15 +338,16 @@ struct Tilt {
 // The window sums D of one unit (see the top), referred to each row's lo (up: to the first position
 // of the last step, lo + walk_end(W)).  Lane (g = lane / 4, q = lane % 4) owns row g of the unit (rv)
 // for X, and outputs kap g and g + 8 of each row tile of columns 2q, 2q + 1.
-__device__ __forceinline__ bool long_window(int W, float c) {  // so much longer than a smooth potential's
-  return (float)W * (float)W * c > 900.f;                 // (about 210) that it is likely to span a gap
-}
+// So much longer than a smooth potential's (about 210) that it is likely to span a gap.  (us per pass, split
+// BF16, line at 450 / 900 / 1800: 1024^2 eps 209 19.3 / 18.7 / 18.1, 2048^2 eps 839 58.4 / 56.7 / 56.6, 576^2 eps 60
+// 14.8 / 14.7 / 13.5: a little high does no harm.)
+__device__ __forceinline__ bool long_window(int W, float c) { return (float)W * (float)W * c > 900.f; }
 __device__ __forceinline__ int walk_end(int W) { return ((W + 31) >> 5) * 32 - 16; }
 // PLAIN: the common case, rows staged, walking down, no look for empty turns (fewer registers).
 template <int FORM, int TN, bool PLAIN>
 __device__ __forceinline__ void window_product(const BandArgs& a, float kc, const RowView& rv, int W, bool up_,
-                                               const Tilt<FORM>& tilt, f32x2 (&D)[TN < 16 ? 1 : TN / 16][2]) {
-  constexpr int MT = TN < 16 ? 1 : TN / 16;
+                                               const Tilt<FORM>& tilt, f32x2 (&D)[TN / 16][2]) {
+  constexpr int MT = TN / 16;
   constexpr int NH = Tilt<FORM>::NH;
   const int q = threadIdx.x & 3;
   const float c = a.c;
@@ -383,7 +378,7 @@ __device__ __forceinline__ void window_product(const BandArgs& a, float kc, cons
     for (int h = 0; h < 2; ++h) {
       G[t][h] = tilt.G[t][h];
       if (up) {
-        const float v = a.step[16 - (16 * t - TN / 2 + (int)((threadIdx.x & 31) >> 2) + (TN < 16 ? 0 : 8 * h))];
+        const float v = a.step[16 - (16 * t - TN / 2 + (int)((threadIdx.x & 31) >> 2) + 8 * h)];
         G[t][h] = pack2(v, v);
       }
     }
@@ -482,9 +477,9 @@ __device__ __forceinline__ void window_product(const BandArgs& a, float kc, cons
 // al[u] + t[i][u].  False, with nothing written, when one is not finite where its row has mass
 // (warp-uniform).
 template <int MODE, int TN>
-__device__ __forceinline__ bool write_unit(const BandArgs& a, int r0, int k0, const float (&al)[TN < 16 ? 1 : TN / 8][2],
-                                           const float (&t)[TN < 16 ? 1 : TN / 8][2], bool skip) {
-  constexpr int NO = TN < 16 ? 1 : TN / 8;                // groups of up to 8 outputs
+__device__ __forceinline__ bool write_unit(const BandArgs& a, int r0, int k0, const float (&al)[TN / 8][2],
+                                           const float (&t)[TN / 8][2], bool skip) {
+  constexpr int NO = TN / 8;                // groups of 8 outputs
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int rA = r0 + 2 * q;
   const size_t y0 = (size_t)(k0 + g) * a.n_rows + rA;
@@ -554,8 +549,8 @@ constexpr int kLongWalk = 320;
 // log-sums of the sums D (referred to lo, or up: lo + walk_end(W)): offset and rest of every output
 template <int FORM, int TN>
 __device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowView& rv, int W, bool up,
-                                         const f32x2 (&D)[TN < 16 ? 1 : TN / 16][2], float (&al)[TN < 16 ? 1 : TN / 8][2],
-                                         float (&t)[TN < 16 ? 1 : TN / 8][2]) {
+                                         const f32x2 (&D)[TN / 16][2], float (&al)[TN / 8][2],
+                                         float (&t)[TN / 8][2]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -563,7 +558,7 @@ __device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowV
     const int at = __shfl_sync(0xffffffffu, rv.lo, 8 * q + 4 * u) + (up ? walk_end(W) : 0);
     const float mr = (float)at - kc;                      // reference - kc
 #pragma unroll
-    for (int i = 0; i < (TN < 16 ? 1 : TN / 8); ++i) {
+    for (int i = 0; i < TN / 8; ++i) {
       const float kap = (float)(8 * i - TN / 2 + g);
       float v[2];
       unpack2(D[i >> 1][i & 1], v[0], v[1]);
@@ -574,7 +569,7 @@ __device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowV
     if (W > kLongWalk) {
       const float walk = (float)(__shfl_sync(0xffffffffu, rv.mh, 8 * q + 4 * u) - at);
 #pragma unroll
-      for (int i = 0; i < (TN < 16 ? 1 : TN / 8); ++i) t[i][u] += step_rounding(a, (float)(8 * i - TN / 2 + g), walk, up);
+      for (int i = 0; i < TN / 8; ++i) t[i][u] += step_rounding(a, (float)(8 * i - TN / 2 + g), walk, up);
     }
   }
 }
@@ -584,9 +579,9 @@ __device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowV
 template <int MODE, int FORM, int TN, bool PLAIN>
 __device__ __forceinline__ bool gemm_unit(const BandArgs& a, int r0, int k0, float kc, const RowView& rv, int W, bool up,
                                           const Tilt<FORM>& tilt, bool skip) {
-  f32x2 D[TN < 16 ? 1 : TN / 16][2];
+  f32x2 D[TN / 16][2];
   window_product<FORM, TN, PLAIN>(a, kc, rv, W, up, tilt, D);
-  float al[TN < 16 ? 1 : TN / 8][2], t[TN < 16 ? 1 : TN / 8][2];   // (an empty row has sums 0: log -inf)
+  float al[TN / 8][2], t[TN / 8][2];   // (an empty row has sums 0: log -inf)
   log_sums<FORM, TN>(a, kc, rv, W, !PLAIN && up, D, al, t);
   return write_unit<MODE, TN>(a, r0, k0, al, t, skip);
 }
@@ -693,12 +688,12 @@ __device__ __forceinline__ RowView recentred(const BandArgs& a, const RowView& r
 template <int MODE, int TN>
 __device__ __noinline__ bool segmented_unit(const BandArgs& a, int r0, int k0, const RowView& rv, int W, bool skip,
                                             unsigned long long* terms) {
-  constexpr int NO = TN < 16 ? 1 : TN / 8;
+  constexpr int NO = TN / 8;
   const float kc = (float)(k0 + TN / 2) + a.shift, c = a.c;
   const int L = min((int)(kRangeMax / (2.f * TN * c)) & ~15, 4096);   // TN (D + mh - lo) c <= TN 2 L c
   if (L < 16 || __any_sync(0xffffffffu, isnan(rv.alpha))) return false;   // (a row for exact sums: fot_plan.cuh)
   Tilt<kFormFp32> tilt;
-  tilt.load(a, TN, false);
+  tilt.load(a, TN);
   float A[NO][2], T[NO][2];                               // the sums so far: offset and rest
 #pragma unroll
   for (int i = 0; i < NO; ++i)
@@ -718,7 +713,7 @@ __device__ __noinline__ bool segmented_unit(const BandArgs& a, int r0, int k0, c
     if (!__any_sync(0xffffffffu, r.wl > 0 && r.alpha + gain >= rv.alpha - kCut)) continue;
     const int Ws = __reduce_max_sync(0xffffffffu, r.wl);
     if ((threadIdx.x & 31) == 0) atomicAdd(terms, (unsigned long long)Ws * TN * 8);
-    f32x2 D[TN < 16 ? 1 : TN / 16][2];
+    f32x2 D[TN / 16][2];
     window_product<kFormFp32, TN, false>(a, kc, r, Ws, false, tilt, D);
     float al[NO][2], t[NO][2];
     log_sums<kFormFp32, TN>(a, kc, r, Ws, false, D, al, t);
@@ -738,14 +733,14 @@ __device__ __noinline__ bool segmented_unit(const BandArgs& a, int r0, int k0, c
   return write_unit<MODE, TN>(a, r0, k0, A, T, skip);
 }
 
-// a unit that is not the common case: a narrow tile, rows not staged, a long window, walking up,
+// a unit that is not the common case: rows not staged, a long window, walking up,
 // outside the bound or with sums that left the range of FP32 (walk 2: no product)
 template <int MODE, int FORM, int TN>
 __device__ __forceinline__ void other_unit_of(const BandArgs& a, int r0, int k0, const RowView& rv, int W, int walk,
                                               bool skip, unsigned long long* terms) {
   if (walk != 2) {
     Tilt<FORM> tilt;
-    tilt.load(a, TN, TN >= 16);
+    tilt.load(a, TN);
     if (gemm_unit<MODE, FORM, TN, false>(a, r0, k0, (float)(k0 + TN / 2) + a.shift, rv, W, walk == 1, tilt, skip)) return;
   }
   if (segmented_unit<MODE, TN>(a, r0, k0, rv, W, skip, terms)) return;
@@ -759,10 +754,8 @@ __device__ __noinline__ void other_unit(const BandArgs& a, int r0, int k0, RowVi
                                         unsigned long long* terms) {
   if (a.tile_w == 32)
     other_unit_of<MODE, FORM, 32>(a, r0, k0, rv, W, walk, skip, terms);
-  else if (a.tile_w == 16)
-    other_unit_of<MODE, FORM, 16>(a, r0, k0, rv, W, walk, skip, terms);
   else
-    other_unit_of<MODE, kFormFp32, 8>(a, r0, k0, rv, W, walk, skip, terms);
+    other_unit_of<MODE, FORM, 16>(a, r0, k0, rv, W, walk, skip, terms);
 }
 
 // A warp's unit of the item that its CTA was launched for.
@@ -788,8 +781,8 @@ __device__ __forceinline__ void product_unit(const BandArgs& a, const Unit& u, c
   const int W = __reduce_max_sync(0xffffffffu, rv.wl);
   const int walk = unit_walk(0.5f * (float)a.tile_w, rv, W, a.c);
   if (walk != 2 && lane == 0 && W > 0)
-    atomicAdd(terms + (FORM == kFormFp32 || a.tile_w < 16 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
-  const bool plain = walk == 0 && a.tile_w >= 16 && (rv.staged || W == 0) && !long_window(W, a.c);
+    atomicAdd(terms + (FORM == kFormFp32 ? 0 : 2), (unsigned long long)W * a.tile_w * 8);
+  const bool plain = walk == 0 && (rv.staged || W == 0) && !long_window(W, a.c);
   if (plain) {
     const float kc = (float)(u.k0 + (a.tile_w >> 1)) + a.shift;
     if (a.tile_w == 32 ? gemm_unit<MODE, FORM, 32, true>(a, u.r0, u.k0, kc, rv, W, false, tilt, u.skip)
@@ -888,7 +881,7 @@ __global__ void __launch_bounds__(kWinThreads, FORM == kFormFp32 ? 4 : 5) window
   Tilt<FORM> tilt;
   const bool pairs = MAXP > 2 && a.group == 2;            // (a batch with problems of both kinds)
   if (!open_unit(tab, a, s_x, &s_bar, pairs, u, [&]() {
-        if (a.tile_w >= 16 && !pairs) tilt.load(a, a.tile_w, true);
+        if (!pairs) tilt.load(a, a.tile_w);
       }))
     return;
   unsigned long long* terms = a.terms + 4 * (blockIdx.x & (kTermSlots - 1));

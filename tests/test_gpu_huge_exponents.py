@@ -10,9 +10,9 @@ from fot_testutil import POT_RTOL, assert_pot_close, f32, to_dev, to_np
 pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:invalid value encountered")]
 
 
-# exact windows, 8- and 16-wide products; one kernel and two (516); the last: beyond the plan's sentinel
+# exact windows, 16- and 32-wide products; one kernel and two (516); the last: beyond the plan's sentinel
 @pytest.mark.parametrize("form", ["fp32", "mixed", "dense"])
-@pytest.mark.parametrize("shape,eps,scale", [((40, 36), 1e-3, 1e7), ((40, 36), 8.0, 1e11), ((40, 36), 60.0, 1e13),
+@pytest.mark.parametrize("shape,eps,scale", [((40, 36), 1e-3, 1e7), ((40, 36), 16.0, 1e11), ((40, 36), 200.0, 1e13),
                                              ((9, 516), 1e-3, 1e8), ((9, 516), 60.0, 1e13), ((40, 36), 1.0, 2.5e38)])
 def test_updates_at_huge_exponents(fot_lib, form, shape, eps, scale):
     B = fot_lib

@@ -29,9 +29,9 @@ def _logsum(B, precision, psi, eps):
 
 
 @pytest.mark.parametrize("shape", [(256, 256), (600, 131)])
-@pytest.mark.parametrize("power", [2.5, 4.0, 6.0])
+@pytest.mark.parametrize("power", [3.5, 5.0, 6.0, 7.0])
 def test_products_of_fp32_operands_are_not_biased(fot_lib, shape, power):
-    """8-, 16- and 32-wide tiles, one-kernel and two-kernel passes, against the dense form, which has
+    """16- and 32-wide tiles, one-kernel and two-kernel passes, against the dense form, which has
     the same exponentials and no products.  Bound: the tensor core cuts a step's sum at 24 bits when
     it adds the last two products, 2^-24 on average each, so 2^-23 per pass and 2^-22 in two; the
     operands' parts are rounded and add nothing on average."""
@@ -71,3 +71,19 @@ def test_long_windows_keep_their_precision(fot_lib, shape, precision):
     rms = (got - ref)[near].pow(2).mean().sqrt().item()
     assert near.sum() > 1000
     assert rms <= (2 * 2.0 ** -22 + 2 * 2.0 ** -22 if precision == "fp32" else 2 * (2.0 ** -19 + 2.0 ** -22)), rms
+
+
+@pytest.mark.parametrize("form", ["fp32", "mixed"])
+def test_small_eps_sums_are_exact(fot_lib, form):
+    """eps 8: one exponential per term and output, whatever the form.  Bound on the mean square, natural
+    logarithm: per pass ex2's 2^-22, uniform, over sqrt(4 pi eps) = 10 terms that matter, and the rounding of a
+    log-sum below 4 (2^-23, uniform); both passes, and half as much again for what is not random."""
+    B = fot_lib
+    eps = LOG2E * 2.0 ** 2.5
+    psi = _level_potential((300, 256), eps, 5)
+    got, terms = _logsum(B, {"fp32": B.FOT_FP32, "mixed": B.FOT_MIXED}[form], psi, eps)
+    ref = _exact_logsum(psi, eps)
+    near = ref.abs() < 0.3
+    rms = (got - ref)[near].pow(2).mean().sqrt().item()
+    assert near.sum() > 1000 and terms[0] == 0 and terms[2] == 0
+    assert rms <= 1.5 * math.sqrt(2) * (2.0 ** -22 / math.sqrt(30) + 2.0 ** -23 * math.log(2) / math.sqrt(3)), rms
