@@ -243,9 +243,9 @@ CLASS_KERNELS = {"band_plan_kernel": "band_plan_kernel, small_pass_kernel",
 # must lose its entry (the bench line then reports traffic null).
 NCU_TRAFFIC = {
     ("tc_pass_kernel", 1024, "mixed"): {
-        "bytes": (4.673536e6 + 0.0 + 8.868096e6 + 0.0) / 2,
-        "source": "ncu --set full, one row-pass and one column-pass launch (mean), the beam and targets of "
-                  "perf/cases.py at 1024^2, eps 209; profiles/banded_passes.md"},
+        "bytes": (4.674048e6 + 0.0 + 8.868096e6 + 0.0) / 2,
+        "source": "ncu, one row-pass and one column-pass launch (mean) of the workload's inputs at 1024^2, eps 209; "
+                  "profiles/banded_passes.md"},
 }
 
 

@@ -69,9 +69,9 @@
 // and 6 MMAs (48 tensor cycles per SM quarter), a unit's set-up and outputs about 450.  A loop of
 // 200 iterations at 1024^2 (800 passes, plan and launch gaps included) went from 31.9 to 14.5 ms with
 // split BF16 and from 45.7 to 16.5 ms with FP32 operands (FFMA with the operands through shared memory
-// before); 100 iterations at 2048^2, split BF16, from 39.8 to 21.2 ms; 256^2 annealed from eps 64 to 1
-// over 300 iterations from 41.7 to 11.7 ms (8.9 with the one-kernel passes of fot_small.cuh); 64^2 at eps 1, 200
-// iterations, from 14.5 to 4.6 ms (2.7).
+// before; 17.2 with the operands' parts rounded); 100 iterations at 2048^2, split BF16, from 39.8 to 21.2 ms (21.9 with
+// the step scale's rounding made up for); 256^2 annealed from eps 64 to 1 over 300 iterations from 41.7 to 11.7
+// ms (8.6 with the one-kernel passes of fot_small.cuh); 64^2 at eps 1, 200 iterations, from 14.5 to 4.6 ms (2.7).
 #pragma once
 
 #include "fot_band.cuh"
@@ -86,6 +86,8 @@ constexpr int kWinWarps = 4;
 constexpr int kWinThreads = 32 * kWinWarps;
 constexpr int kPitchCap = 40 * 32 + 16;   // floats staged per row at most (41 KB of 8 rows: five CTAs fit
                                           // an SM); wider spans are read from global memory
+                                          // (2048^2, split BF16, a half-step: eps 6000, most
+                                          // items staged, 172 us, eps 7000, none, 180)
 constexpr int kSpinDefault = 1 << 20;     // polls of a bounded wait
 constexpr int kTiltWords = 2 * 2 * 32;    // uint4 words of a tilt table: 2 row tiles x (hi, lo) x lanes
 
