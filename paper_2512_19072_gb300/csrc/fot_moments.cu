@@ -183,11 +183,12 @@ __device__ __forceinline__ bool moment_unit(const BandArgs& a, int r0, int k0, f
   }
   if (__any_sync(0xffffffffu, bad)) return false;
   if (W > kLongWalk) {
+    const float err = a.step_err[lane], walk = (float)(rv.mh - rv.lo);   // (as log_sums)
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const float walk = (float)(__shfl_sync(0xffffffffu, rv.mh, 8 * q + 4 * u) - lo[u]);
+      const float w = __shfl_sync(0xffffffffu, walk, 8 * q + 4 * u);
 #pragma unroll
-      for (int i = 0; i < 2; ++i) rest[i][u] += step_rounding(a, (float)(8 * i - 8 + g), walk, false);
+      for (int i = 0; i < 2; ++i) rest[i][u] = fmaf(__shfl_sync(0xffffffffu, err, 8 * i + 8 + g), w, rest[i][u]);
     }
   }
   if (skip) return true;

@@ -538,14 +538,12 @@ __device__ __forceinline__ bool write_unit(const BandArgs& a, int r0, int k0, co
   return true;
 }
 
-// What the rounding of the step scale G took from a sum, in log2 units: up to 2^-25 per step, over the steps
-// between the reference and the row's largest term (walk: positions).
-__device__ __forceinline__ float step_rounding(const BandArgs& a, float kap, float walk, bool up) {
-  return a.step_err[16 + (int)(up ? -kap : kap)] * (up ? -walk : walk);
-}
-// Windows from which on that is made up for: below, it is no more than the FP32 error of the rest (log-sums
-// at 1500 x 1400, FP32 form, rms: eps 369 4.7e-7 without and 3.2e-7 with it; eps 5900 1.4e-6 and 3.8e-7),
-// and at 1024^2 and eps 209 a solve takes 5 % longer with it.
+// Windows from which on outputs get back what the rounding of the step scale G took from their sums: up to
+// 2^-25 per step (a.step_err, log2 per position), over the steps between the reference and the row's largest
+// term.  Below, it is no more than the FP32 error of the rest (log-sums at 1500 x 1400, FP32 form, rms: eps 369
+// 4.7e-7 without and 3.2e-7 with it; eps 5900 1.4e-6 and 3.8e-7), and a solve at 1024^2 and eps 209 takes
+// longer with it (with a lane's entries read from the constant bank one by one, 5 %; 100 iterations at 2048^2,
+// split BF16, 20.9 ms without, 21.9 that way, 21.1 with one read and shuffles).
 constexpr int kLongWalk = 320;
 
 // log-sums of the sums D (referred to lo, or up: lo + walk_end(W)): offset and rest of every output
@@ -568,10 +566,17 @@ __device__ __forceinline__ void log_sums(const BandArgs& a, float kc, const RowV
       al[i][u] = alpha;
       t[i][u] = fmaf(fmaf(2.f * kap, mr, -kap * kap), a.c, l2);
     }
-    if (W > kLongWalk) {
-      const float walk = (float)(__shfl_sync(0xffffffffu, rv.mh, 8 * q + 4 * u) - at);
+  }
+  if (W > kLongWalk) {
+    // each lane reads one entry (the constant bank answers one address at a time), shuffles bring the others
+    const float err = a.step_err[up ? 32 - lane : lane];  // of kap = lane - 16
+    const float walk = up ? (float)(rv.lo + walk_end(W) - rv.mh) : (float)(rv.mh - rv.lo);
+    const float w0 = __shfl_sync(0xffffffffu, walk, 8 * q), w1 = __shfl_sync(0xffffffffu, walk, 8 * q + 4);
 #pragma unroll
-      for (int i = 0; i < TN / 8; ++i) t[i][u] += step_rounding(a, (float)(8 * i - TN / 2 + g), walk, up);
+    for (int i = 0; i < TN / 8; ++i) {
+      const float e = __shfl_sync(0xffffffffu, err, 8 * i + g + 16 - TN / 2);
+      t[i][0] = fmaf(e, w0, t[i][0]);
+      t[i][1] = fmaf(e, w1, t[i][1]);
     }
   }
 }
